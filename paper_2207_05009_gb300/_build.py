@@ -44,8 +44,7 @@ def _stale(target, inputs):
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
     """Compile every csrc/*.cu in parallel, then link libplo.so.  Extra nvcc
-    flags (for example -DPLO_RENDER_MIN_BLOCKS=3) come from $PLO_NVCC_FLAGS;
-    pass force=True after changing them."""
+    flags come from $PLO_NVCC_FLAGS; pass force=True after changing them."""
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
     deps = _deps()

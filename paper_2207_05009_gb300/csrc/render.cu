@@ -11,16 +11,28 @@
 // iteration.  Child slots come from the bits of the point's integer
 // coordinates on the finest grid.
 //
-// Numerics (all FP32, no FP64 on the device):
-//   * The ray position is kept as an unevaluated sum hi + lo of two floats
-//     per axis ("double-float").  Segment lengths come from exact dyadic cell
-//     planes minus that position, so every segment length has ~1e-7 relative
+// What bounds it: the latency of the dependent node loads, then instruction
+// issue (65% of the issue slots, depth-9 luminaire, 2M rays), at a tenth of
+// the DRAM bandwidth.  So the walk is built to need few instructions per cell
+// and little shared memory (what is left is L1): fixed-point plane parameters
+// (below), no staging of the top nodes (the test for it cost more than the
+// L1 hits it saved: 18.7 against 16.5 ms for 9M rays at depth 9), and SH
+// emission evaluated for 32 leaves at a time from a per-warp queue (walk_rays).
+// Before, with double-float positions, staged top nodes and the emission
+// evaluated where a ray meets it (9M rays at depth 9, FP32 leaves / 2M at
+// depth 8, BF16 leaves, T < 1e-4 stop): 18.4 / 2.95 ms; now 12.7 / 1.95 ms.
+//
+// Numerics (no FP64 on the device):
+//   * Each axis is mirrored so that the ray goes up it.  The parameter at
+//     which a ray crosses a plane of the finest grid is a 64-bit fixed-point
+//     number, linear in the plane's index, set up once per ray in
+//     double-float arithmetic (pairs of floats, ~2^-46).  Segment lengths are
+//     differences of such parameters, so every length has ~1e-7 relative
 //     error however far the ray origin is, and the cell sequence matches an
 //     FP64 walk except for rays passing within ~1e-13 of a cell edge.
-//   * The exit coordinate is snapped onto the exact plane; the next cell is
-//     found by re-descending from the deepest common ancestor (kept on a
-//     per-ray stack) with the tie rule "on a plane, go where the direction
-//     points", so progress is guaranteed.
+//   * The next cell is found by re-descending from the deepest common
+//     ancestor (kept on a per-ray stack) with the tie rule "on a plane, go
+//     where the direction points", so progress is guaranteed.
 //   * Optical depth is accumulated as a compensated (two-float) sum;
 //     T = exp(-OD) or max(0, 1 - OD) is recomputed from it after each leaf.
 #include <cuda_bf16.h>
@@ -39,17 +51,13 @@ namespace plo {
 namespace {
 
 constexpr int BLOCK = 256;
-#ifndef PLO_RENDER_MIN_BLOCKS
-#define PLO_RENDER_MIN_BLOCKS 4  // resident blocks per SM the register budget is sized for (measured best)
-#endif
-#ifndef PLO_BRICK_MIN_BLOCKS
-#define PLO_BRICK_MIN_BLOCKS 3  // the same for the brick-layout kernels
-#endif
 constexpr int WARPS = BLOCK / 32;
 constexpr int64_t RENDER_CLAIM = 32;  // rays a warp claims at a time from the shared cursor (32 measured best of 32-128)
-#ifndef PLO_DESCEND_LEVELS
-#define PLO_DESCEND_LEVELS 4  // tree levels a descent goes down per step (measured best of 2, 3, 4, 5, all)
-#endif
+constexpr int DESCEND_LEVELS = 4;  // tree levels a descent goes down per step (measured best of 2, 3, 4, 5, 6)
+// Lanes without a ray that wait for each other before they take new ones: ray
+// setup is about 900 instructions however few lanes run it (4, 6, 8 lanes,
+// 9M rays of the depth-9 luminaire: 12.89, 12.75, 12.67 ms).
+constexpr int REFILL = 8;
 
 // One packed tree as the kernels see it.
 struct TreeParams {
@@ -77,6 +85,7 @@ struct KParams {
     float sphere[4];  // sphere proxy: centre, radius (world space)
     const float* rays;
     unsigned long long* cursor;  // shared claim counter (NULL: static chunks per warp)
+    int64_t claim;               // rays a warp claims from it at a time
     int64_t n;
     int64_t chunk;  // rays per warp
     float* rgb;
@@ -111,12 +120,15 @@ __device__ __forceinline__ DF df_mul(DF a, float rh, float rl) {
     e = __fmaf_rn(a.lo, rh, e);
     return fast_two_sum(p, e);
 }
-// double-float reciprocal of d = dh + dl (dh finite, non-zero)
+// double-float reciprocal of d = dh + dl (0 < dh <= 1; infinite or NaN where 1/d overflows)
 __device__ __forceinline__ void df_recip(float dh, float dl, float& rh, float& rl) {
-    rh = __frcp_rn(dh);
-    float r = __fmaf_rn(-rh, dh, 1.0f);  // exact residual of the rounded reciprocal
+    asm("rcp.approx.f32 %0, %1;" : "=f"(rh) : "f"(dh));
+    float r = __fmaf_rn(-rh, dh, 1.0f);  // residual of the approximate reciprocal (exact)
     r = __fmaf_rn(-rh, dl, r);
-    rl = __fmul_rn(r, rh);
+    r = __fmul_rn(r, rh);
+    const float h = __fadd_rn(rh, r);
+    rl = __fsub_rn(r, __fsub_rn(h, rh));
+    rh = h;
 }
 // p + t * d, all double-float
 __device__ __forceinline__ DF df_axpy(DF p, DF t, float dh, float dl) {
@@ -169,24 +181,32 @@ __device__ __forceinline__ DF df_from_plane(float P, DF p) {
 __device__ __forceinline__ bool df_less(DF a, DF b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
 __device__ __forceinline__ bool df_eq(DF a, DF b) { return a.hi == b.hi && a.lo == b.lo; }
 __device__ __forceinline__ float pow2i(int e) { return __int_as_float((127 + e) << 23); }  // e in [-126, 127]
-// Finest-grid coordinate of p (depth D, scale = 2^D): floor(p 2^D), except
-// that a point exactly on a grid plane belongs to the cell below it when the
-// direction is negative (the tie rule), clamped to [0, 2^D - 1] (the root box
-// is closed).  Bit D-1-l of the result is the child bit at level l: the same
-// decision as comparing p with every mid-plane on the way down.
-__device__ __forceinline__ uint32_t quantize(DF p, float scale, uint32_t qmax, float d) {
+// Finest-grid coordinate of p on a mirrored axis (depth D, scale = 2^D):
+// floor(p 2^D), clamped to [0, 2^D - 1] (the root box is closed).  A point on
+// a grid plane belongs to the cell the ray goes into: the one above it, which
+// on a mirrored axis is the one below it in the caller's coordinates (the tie
+// rule).  Bit D-1-l of the result is the child bit at level l.
+__device__ __forceinline__ uint32_t quantize(DF p, float scale, uint32_t qmax) {
     const float h = p.hi * scale;  // exact: scale is a power of two
     const float f = floorf(h);
     int q = (int)f;
-    if (h == f && (p.lo < 0.0f || (p.lo == 0.0f && d < 0.0f))) --q;
+    if (h == f && p.lo < 0.0f) --q;
     q = max(q, 0);
     return min((uint32_t)q, qmax);
 }
 
-// Loads one SH record and returns sum_k c_{ch,k} Y_k for the three channels.
+template <int PREC>
+__device__ __forceinline__ float decode_sigma(uint32_t y, int prec) {
+    if (PREC == PLO_PREC_FP32 || (PREC < 0 && prec == PLO_PREC_FP32)) return __uint_as_float(y);
+    return __uint_as_float((y & 0xFFFFFFu) << 7);  // 24-bit float: exponent + 16 mantissa bits
+}
+
+// ---------------------------------------------------------------- SH emission
+// sum_k c_{ch,k} Y_k(dir) of the three channels of one record.
 template <int K, int PREC>
-__device__ __forceinline__ void sh_eval(const uint8_t* rec, uint32_t yword, const float* Y, float& r, float& g,
-                                        float& b) {
+__device__ __forceinline__ void sh_eval(const uint8_t* rec, const float* dir, float& r, float& g, float& b) {
+    float Y[K];
+    sh_basis<K>(dir[0], dir[BLOCK], dir[2 * BLOCK], Y);
     float acc[3] = {0.0f, 0.0f, 0.0f};
     if (PREC == PLO_PREC_FP32) {
         constexpr int NV = (3 * K + 3) / 4;
@@ -219,50 +239,31 @@ __device__ __forceinline__ void sh_eval(const uint8_t* rec, uint32_t yword, cons
                 }
             }
         }
-        float s = pow2i((int)(yword >> 24) - 127);
-        acc[0] *= s;
-        acc[1] *= s;
-        acc[2] *= s;
     }
     r = acc[0];
     g = acc[1];
     b = acc[2];
 }
 
-template <int PREC>
-__device__ __forceinline__ float decode_sigma(uint32_t y, int prec) {
-    if (PREC == PLO_PREC_FP32 || (PREC < 0 && prec == PLO_PREC_FP32)) return __uint_as_float(y);
-    return __uint_as_float((y & 0xFFFFFFu) << 7);  // 24-bit float: exponent + 16 mantissa bits
-}
-
-// SH emission of one record; K / PREC given at compile time, or read from
-// the tree when K == 0 (the batch kernel mixes trees).
+// The same with K / PREC given at compile time, or read from the tree when
+// K == 0 (the batch kernel mixes trees).
 template <int K, int PREC>
-__device__ __forceinline__ void sh_emission(const TreeParams& tp, uint32_t rec, uint32_t yword, const float* dirn,
-                                            float& r, float& g, float& b, const float* sY = nullptr) {
+__device__ __forceinline__ void sh_record(const TreeParams& tp, uint32_t rec, const float* dir, float& r, float& g,
+                                          float& b) {
     const uint8_t* p = tp.sh + (size_t)rec * tp.sh_stride;
-    if (K > 0) {  // the per-lane basis in shared memory (sY, set at the ray's start)
-        float Y[K > 0 ? K : 1];
-#pragma unroll
-        for (int k = 0; k < (K > 0 ? K : 1); ++k) Y[k] = sY[k * BLOCK];
-        sh_eval<(K > 0 ? K : 1), PREC>(p, yword, Y, r, g, b);
-        return;
-    }
-    // each degree builds only its own basis, so that the registers of the
-    // larger bases are taken only in their branches
-#define PLO_SH_CASE(KK, PP)                                  \
-    if (tp.K == KK && tp.prec == PP) {                       \
-        float Y[KK];                                         \
-        sh_basis<KK>(dirn[0], dirn[1], dirn[2], Y);          \
-        return sh_eval<KK, PP>(p, yword, Y, r, g, b);        \
-    }
-    PLO_SH_CASE(16, PLO_PREC_FP32) PLO_SH_CASE(9, PLO_PREC_FP32) PLO_SH_CASE(16, PLO_PREC_FP16)
-    PLO_SH_CASE(9, PLO_PREC_FP16) PLO_SH_CASE(16, PLO_PREC_BF16) PLO_SH_CASE(9, PLO_PREC_BF16)
-    PLO_SH_CASE(4, PLO_PREC_FP32) PLO_SH_CASE(4, PLO_PREC_FP16) PLO_SH_CASE(4, PLO_PREC_BF16)
-    PLO_SH_CASE(1, PLO_PREC_FP32) PLO_SH_CASE(1, PLO_PREC_FP16) PLO_SH_CASE(1, PLO_PREC_BF16)
-    PLO_SH_CASE(25, PLO_PREC_FP32) PLO_SH_CASE(25, PLO_PREC_FP16) PLO_SH_CASE(25, PLO_PREC_BF16)
+    if constexpr (K > 0) {
+        sh_eval<K, PREC>(p, dir, r, g, b);
+    } else {
+#define PLO_SH_CASE(KK, PP) \
+    if (tp.K == KK && tp.prec == PP) return sh_eval<KK, PP>(p, dir, r, g, b);
+        PLO_SH_CASE(16, PLO_PREC_FP32) PLO_SH_CASE(9, PLO_PREC_FP32) PLO_SH_CASE(16, PLO_PREC_FP16)
+        PLO_SH_CASE(9, PLO_PREC_FP16) PLO_SH_CASE(16, PLO_PREC_BF16) PLO_SH_CASE(9, PLO_PREC_BF16)
+        PLO_SH_CASE(4, PLO_PREC_FP32) PLO_SH_CASE(4, PLO_PREC_FP16) PLO_SH_CASE(4, PLO_PREC_BF16)
+        PLO_SH_CASE(1, PLO_PREC_FP32) PLO_SH_CASE(1, PLO_PREC_FP16) PLO_SH_CASE(1, PLO_PREC_BF16)
+        PLO_SH_CASE(25, PLO_PREC_FP32) PLO_SH_CASE(25, PLO_PREC_FP16) PLO_SH_CASE(25, PLO_PREC_BF16)
 #undef PLO_SH_CASE
-    r = g = b = 0.0f;
+        r = g = b = 0.0f;
+    }
 }
 
 __device__ __forceinline__ float act_fn(float s, int act, float l_max) {
@@ -270,88 +271,101 @@ __device__ __forceinline__ float act_fn(float s, int act, float l_max) {
 }
 
 // ---------------------------------------------------------------- per-ray state
-// Lane states: idle (no ray), descending to the cell at its current point,
-// at a leaf cell waiting to composite it, or walking a brick cell by cell.
-enum : int { ST_IDLE = 0, ST_DESCEND = 1, ST_LEAF = 2, ST_BRICK = 3 };
+// Lane states: idle (no ray), finished (emission still queued, outputs not
+// written; _LIMIT: stopped by the step limit), descending to the cell at its
+// current point, or at a leaf cell waiting to composite it.
+enum : int { ST_IDLE = 0, ST_DONE = 1, ST_DONE_LIMIT = 2, ST_DESCEND = 3, ST_LEAF = 4 };
+
+// The walk's ray parameter is a 64-bit fixed-point number with T_FRAC
+// fractional bits.  It counts from the point where the ray enters the proxy,
+// in units that make the largest unit-cube direction component lie in
+// [1/2, 1) (a power-of-two scaling of the caller's parameter), so it stays
+// below 2.  Every axis is mirrored where the direction is negative, so the
+// walk only ever goes up: the exit planes of a cell are its upper faces.
+constexpr int T_FRAC = 60;
+constexpr long long T_CAP = 5ll << (T_FRAC - 1);  // 2.5: the parameter of a plane the ray never reaches
+// Two planes crossed within 2^-44 of each other are crossed together, so that
+// a ray through a shared edge or corner goes through it in one step instead
+// of leaving a sliver segment behind.
+constexpr long long T_TIE = 1ll << (T_FRAC - 44);
+constexpr float FLAT = 1.0e30f;  // 1 / direction above which an axis counts as parallel to its planes
 
 struct Ray {
-    DF p[3];
-    float d[3];         // unit-cube direction (high part; the low part is in low_parts())
-    float dirn[3];      // normalised world direction for the SH basis
+    long long t;              // parameter of the current cell's entry
+    uint32_t q[3];            // current point on the mirrored finest (depth-D) grid
+    float scale;              // caller's parameter per unit of t (a power of two)
+    uint32_t flip;            // bit a: axis a is mirrored (= the child-slot bits to flip)
     float T, r, g, b;
     DF od;
-    DF t;               // ray parameter at the current cell entry (trace only)
-    DF rem;             // ray parameter left inside the sphere proxy (sphere only)
-    uint32_t q[3];      // integer coordinates of the current point on the finest (depth-D) grid
-                        // (ST_BRICK: of the point where the ray entered the brick)
-    uint32_t node;      // node whose child is looked up next (ST_DESCEND); the brick (ST_BRICK)
-    DF tn[3];           // ST_BRICK: ray parameter, from the brick entry point, of the next
-                        // finest-grid plane crossed on each axis
-    DF tb;              // ST_BRICK: the same parameter at the current cell's entry
-    uint32_t loc;       // ST_BRICK: brick-local finest coordinates x | y << 4 | z << 8
+    DF t0;           // caller's parameter at t = 0 (trace only)
+    long long tend;  // parameter where the ray leaves the sphere proxy (sphere only)
+    uint32_t node;   // node whose child is looked up next (ST_DESCEND); the brick while in one
     uint32_t entry_x, entry_y;
     int level;
     int steps;
-    int slot;           // slot of the current cell in its parent (trace only)
     int state;
-    int status;
-    int tree;           // index into the batch's tree table (batch kernel only)
+    int brick;  // the current cell is a finest cell of brick `node`
+    int tree;   // index into the batch's tree table (batch kernel only)
 };
 
-// Per-ray constants read once per cell, kept in shared memory to leave
-// registers to the hot state: the low-order part of the double-float
-// direction (dl, zero for the unit box) at [a * BLOCK], the reciprocal 1/d
-// as a double-float, low part rl at [(3 + a) * BLOCK] and high part rh at
-// [(6 + a) * BLOCK].  Column per thread.
-__device__ __forceinline__ float* low_parts() {
-    __shared__ float s_low[9 * BLOCK];
-    return s_low + threadIdx.x;
+// What a ray keeps per axis from its start to its end, in shared memory, a
+// column per thread: registers for it would cost a resident block per SM or
+// spills (depth-9 luminaire, 9M rays: 12.9 ms; 13.9 with the 31-bit values in
+// registers, 16.3 with everything in registers and 3 blocks).
+//
+// Finest-grid plane k of the axis lies at parameter A + min(k, kmax) B (mod
+// 2^64): one 64-bit multiply-add, the same value whatever the cell it bounds.
+// kmax is the first plane behind the ray's end, which keeps the product in
+// range however flat the ray is on that axis.  The position is o31 + t d32
+// with 31 fractional bits, rounded down.
+struct AxisShared {
+    ulonglong2 plane[3 * BLOCK];  // A, B
+    uint2 pos[3 * BLOCK];         // o31, d32
+    uint32_t kmax[3 * BLOCK];
+};
+__device__ __forceinline__ AxisShared& axes() {
+    __shared__ AxisShared s;
+    return s;
+}
+__device__ __forceinline__ long long plane_at(int a, uint32_t k) {
+    const ulonglong2 v = axes().plane[a * BLOCK + threadIdx.x];
+    return (long long)(v.x + (unsigned long long)min(k, axes().kmax[a * BLOCK + threadIdx.x]) * v.y);
 }
 
-__device__ __forceinline__ uint2 load_entry(const TreeParams& tp, const uint2* s_nodes, uint32_t node, int slot) {
-    if (node < (uint32_t)tp.n_top) return s_nodes[tp.s_off + node * 8 + slot];
+// A double-float in [0, 4) as a walk parameter.
+__device__ __forceinline__ long long to_fixed(DF v) {
+    const float s = 1152921504606846976.0f;  // 2^T_FRAC
+    return __float2ll_rn(v.hi * s) + __float2ll_rn(v.lo * s);
+}
+
+__device__ __forceinline__ uint2 load_entry(const TreeParams& tp, const uint2* s_nodes, uint32_t node, uint32_t slot) {
+    if (s_nodes && node < (uint32_t)tp.n_top) return s_nodes[tp.s_off + node * 8 + slot];
     return __ldg(tp.nodes + (size_t)node * 8 + slot);
 }
 
-// Brick-local cell index: Morton interleave of the local coordinates
-// (loc = x | y << 4 | z << 8, each < 8), x lowest.
+// Entry of the finest cell R.q of a brick: index = Morton interleave of the
+// brick-local coordinates (mirrored back), x lowest.
 __device__ __forceinline__ uint32_t spread3(uint32_t x) { return (x & 1u) | ((x & 2u) << 2) | ((x & 4u) << 4); }
-__device__ __forceinline__ uint2 brick_entry(const TreeParams& tp, uint32_t brick, uint32_t loc) {
-    const uint32_t m = spread3(loc & 15u) | (spread3((loc >> 4) & 15u) << 1) | (spread3(loc >> 8) << 2);
-    return __ldg(tp.bricks + ((size_t)brick << (3 * tp.brick_log)) + m);
-}
-
-// Enters brick `brick`, the level-top_depth cell that holds the current
-// point: the brick-local coordinates of the finest cell R.q, and per axis the
-// parameter of the next finest plane from the current point,
-// (P - p) / d in double-float (as the octree step computes its exits).  The
-// first cell's entry is loaded here, for the next iteration.
-__device__ __forceinline__ void brick_enter(const TreeParams& tp, Ray& R, uint32_t brick) {
+__device__ __forceinline__ void load_brick(const TreeParams& tp, Ray& R) {
     const uint32_t smask = (1u << tp.brick_log) - 1u;
-    R.node = brick;
-    R.loc = (R.q[0] & smask) | ((R.q[1] & smask) << 4) | ((R.q[2] & smask) << 8);
-    const float cell = pow2i(-tp.depth);
+    uint32_t m = 0;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        DF v = {INFINITY, 0.0f};
-        if (R.d[a] != 0.0f) {
-            const float P = (float)(R.q[a] + (R.d[a] > 0.0f ? 1u : 0u)) * cell;  // exact
-            v = df_mul(df_from_plane(P, R.p[a]), low_parts()[(6 + a) * BLOCK], low_parts()[(3 + a) * BLOCK]);
-            if (v.hi < 0.0f) v = {0.0f, 0.0f};
-        }
-        R.tn[a] = v;
-    }
-    R.tb = {0.0f, 0.0f};
-    const uint2 e = brick_entry(tp, brick, R.loc);
+    for (int a = 0; a < 3; ++a)
+        m |= spread3((R.q[a] ^ ((R.flip >> a) & 1u ? smask : 0u)) & smask) << a;
+    const uint2 e = __ldg(tp.bricks + ((size_t)R.node << (3 * tp.brick_log)) + m);
     R.entry_x = e.x;
     R.entry_y = e.y;
-    R.state = ST_BRICK;
+}
+
+// Child slot, at the level `sh` bits above the finest one, of the point R.q.
+__device__ __forceinline__ uint32_t child_slot(const Ray& R, int sh) {
+    return (((R.q[0] >> sh) & 1u) | (((R.q[1] >> sh) & 1u) << 1) | (((R.q[2] >> sh) & 1u) << 2)) ^ R.flip;
 }
 
 // Descends from R.node (level R.level) towards the leaf or empty octant that
 // holds the point, taking the child bits from the finest-grid coordinates
-// R.q, and ends in ST_LEAF (or, in the brick layout, in ST_BRICK when it
-// reaches a brick).  A step goes down at most PLO_DESCEND_LEVELS levels; a
+// R.q, and ends in ST_LEAF (in the brick layout also at a finest cell of the
+// brick it reaches).  A step goes down at most DESCEND_LEVELS levels; a
 // longer descent goes on in the next step while the other lanes composite.
 // A lane needs 2 levels per step on average but the warp ran the longest
 // descent among its lanes, 5.7 levels (depth-10 luminaire, 16M room rays):
@@ -359,20 +373,31 @@ __device__ __forceinline__ void brick_enter(const TreeParams& tp, Ray& R, uint32
 // 397 with FP16; 2 levels gained nothing and 1 level lost.
 template <bool BRICKS, int PREC>
 __device__ __forceinline__ void descend_step(const TreeParams& tp, const uint2* s_nodes, Ray& R, uint32_t* stack) {
-    for (int guard = 0; guard < PLO_DESCEND_LEVELS; ++guard) {
-        const int sh = tp.depth - 1 - R.level;
-        R.slot = (int)(((R.q[0] >> sh) & 1u) | (((R.q[1] >> sh) & 1u) << 1) | (((R.q[2] >> sh) & 1u) << 2));
-        uint2 e = load_entry(tp, s_nodes, R.node, R.slot);
+    // the child bits of the levels to come, at the top of a word per axis
+    uint32_t x[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        x[a] = (R.q[a] ^ ((R.flip >> a) & 1u ? 0xFFFFFFFFu : 0u)) << (32 - tp.depth + R.level);
+    for (int guard = 0; guard < DESCEND_LEVELS; ++guard) {
+        uint32_t slot = x[2] >> 31;
+        slot = __funnelshift_l(x[1], slot, 1);
+        slot = __funnelshift_l(x[0], slot, 1);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) x[a] <<= 1;
+        uint2 e = load_entry(tp, s_nodes, R.node, slot);
         ++R.level;
         if ((e.x & LEAF_BIT) || R.level >= tp.top_depth) {  // leaf, empty octant, brick (or a malformed table)
+            R.state = ST_LEAF;
             if (BRICKS && tp.bricks && !(e.x & LEAF_BIT) && R.level == tp.top_depth) {
-                brick_enter(tp, R, e.x);
+                R.node = e.x;
+                R.brick = 1;
+                R.level = tp.depth;
+                load_brick(tp, R);
                 return;
             }
             if (!(e.x & LEAF_BIT)) e = make_uint2(ENTRY_EMPTY, 0u);
             R.entry_x = e.x;
             R.entry_y = e.y;
-            R.state = ST_LEAF;
             // the SH record is read in the next iteration: start pulling it
             // into L2 now, for 16-bit records (measured on the depth-10
             // workload: FP16 427 -> 436 Mrays/s with it, FP32 410 -> 404,
@@ -394,19 +419,20 @@ __device__ __forceinline__ void descend_step(const TreeParams& tp, const uint2* 
     }
 }
 
-__device__ __forceinline__ void ray_store(const KParams& kp, int64_t i, const Ray& R) {
+__device__ __forceinline__ void ray_store(const KParams& kp, int64_t i, const Ray& R, int status = PLO_RAY_OK) {
     kp.rgb[3 * i + 0] = R.r;
     kp.rgb[3 * i + 1] = R.g;
     kp.rgb[3 * i + 2] = R.b;
     kp.T[i] = kp.saturate && R.T < kp.t_stop ? 0.0f : R.T;  // a saturated ray is opaque (Sec. 6.2)
-    if (kp.status) kp.status[i] = R.status;
+    if (kp.status) kp.status[i] = status;
     if (kp.tr_count) kp.tr_count[i] = R.steps;
 }
 
-// Proxy clip.  On a hit the lane enters ST_DESCEND at the root; on a miss or
+// Proxy clip.  On a hit the lane enters ST_DESCEND at the root and the
+// normalised world direction (for the SH basis) is left in dir; on a miss or
 // an invalid ray the outputs are written and the lane stays ST_IDLE.
 template <bool TRACE, bool SPHERE>
-__device__ void ray_begin(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R, uint32_t* stack) {
+__device__ void ray_begin(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R, uint32_t* stack, float* dir) {
     const float* q = kp.rays + 6 * i;
     float o[3], dw[3];
 #pragma unroll
@@ -417,54 +443,55 @@ __device__ void ray_begin(const KParams& kp, const TreeParams& tp, int64_t i, Ra
     R.T = 1.0f;
     R.r = R.g = R.b = 0.0f;
     R.od = {0.0f, 0.0f};
-    R.t = {0.0f, 0.0f};
-    R.status = PLO_RAY_OK;
     R.steps = 0;
     R.state = ST_IDLE;
     bool bad = dw[0] == 0.0f && dw[1] == 0.0f && dw[2] == 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) bad |= !isfinite(o[a]) || !isfinite(dw[a]);
     if (bad) {
-        R.status = PLO_RAY_INVALID;
         R.r = R.g = R.b = R.T = __int_as_float(0x7fc00000);
-        ray_store(kp, i, R);
+        ray_store(kp, i, R, PLO_RAY_INVALID);
         return;
     }
     const float inv_n = rsqrtf(__fadd_rn(__fadd_rn(__fmul_rn(dw[0], dw[0]), __fmul_rn(dw[1], dw[1])),
                                          __fmul_rn(dw[2], dw[2])));
-    DF ou[3];  // origin in unit-cube coordinates, (o - bmin) / extent in double-float
+    // origin and direction in unit-cube coordinates, (o - bmin) / extent in
+    // double-float; the direction then scaled by 2^-e
+    DF m[3], du[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        R.dirn[a] = __fmul_rn(dw[a], inv_n);
-        ou[a] = df_mul(two_sum(o[a], -tp.bmin[a]), tp.inv_ext[a], tp.inv_ext_lo[a]);
-        DF du = df_mul(DF{dw[a], 0.0f}, tp.inv_ext[a], tp.inv_ext_lo[a]);
-        R.d[a] = du.hi;
-        low_parts()[a * BLOCK] = du.lo;
+        if (!TRACE) dir[a * BLOCK] = __fmul_rn(dw[a], inv_n);
+        m[a] = df_mul(two_sum(o[a], -tp.bmin[a]), tp.inv_ext[a], tp.inv_ext_lo[a]);
+        du[a] = df_mul(DF{dw[a], 0.0f}, tp.inv_ext[a], tp.inv_ext_lo[a]);
     }
-    // slab test in double-float
+    const float dmax = fmaxf(fabsf(du[0].hi), fmaxf(fabsf(du[1].hi), fabsf(du[2].hi)));
+    const int e = max(-125, min(126, (int)(__float_as_uint(dmax) >> 23) - 126));
+    const float up = pow2i(e);
+    R.scale = pow2i(-e);
+    // slab test in double-float, on mirrored axes (the ray goes up): it enters
+    // by the faces at 0 and leaves by those at 1
+    R.flip = 0u;
     DF tn = {-INFINITY, 0.0f}, tf = {INFINITY, 0.0f};
-    DF near_a[3];
+    DF near_a[3], rd[3];  // rd: 1 / direction
     bool miss = false;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
+        if (du[a].hi < 0.0f) {
+            R.flip |= 1u << a;
+            du[a] = df_neg(du[a]);
+            m[a] = df_from_plane(1.0f, m[a]);
+        }
+        du[a].hi *= R.scale;
+        du[a].lo *= R.scale;
         near_a[a] = {-INFINITY, 0.0f};
-        if (R.d[a] == 0.0f) {
-            if (ou[a].hi < 0.0f || ou[a].hi > 1.0f || (ou[a].hi == 0.0f && ou[a].lo < 0.0f) ||
-                (ou[a].hi == 1.0f && ou[a].lo > 0.0f))
-                miss = true;
+        df_recip(du[a].hi, du[a].lo, rd[a].hi, rd[a].lo);
+        if (!(rd[a].hi < FLAT)) {  // (nearly) parallel to the slab: never crosses a plane
+            miss |= m[a].hi < 0.0f || m[a].hi > 1.0f || (m[a].hi == 0.0f && m[a].lo < 0.0f) ||
+                    (m[a].hi == 1.0f && m[a].lo > 0.0f);
             continue;
         }
-        float rh, rl;
-        df_recip(R.d[a], low_parts()[a * BLOCK], rh, rl);
-        low_parts()[(6 + a) * BLOCK] = rh;
-        low_parts()[(3 + a) * BLOCK] = rl;
-        DF t0 = df_mul(df_from_plane(0.0f, ou[a]), rh, rl);
-        DF t1 = df_mul(df_from_plane(1.0f, ou[a]), rh, rl);
-        if (df_less(t1, t0)) {
-            DF s = t0;
-            t0 = t1;
-            t1 = s;
-        }
+        const DF t0 = df_mul(df_neg(m[a]), rd[a].hi, rd[a].lo);
+        const DF t1 = df_mul(df_from_plane(1.0f, m[a]), rd[a].hi, rd[a].lo);
         near_a[a] = t0;
         if (df_less(tn, t0)) tn = t0;
         if (df_less(t1, tf)) tf = t1;
@@ -500,7 +527,9 @@ __device__ void ray_begin(const KParams& kp, const TreeParams& tp, int64_t i, Ra
         const DF m = df_neg(b.hi >= 0.0f ? df_add(b, sq) : df_sub(b, sq));
         const DF r_far = df_div(m, a2), r_near = df_div(q, m);
         const bool mneg = m.hi < 0.0f;
-        const DF s0 = mneg ? r_far : r_near, s1 = mneg ? r_near : r_far;
+        DF s0 = mneg ? r_far : r_near, s1 = mneg ? r_near : r_far;
+        s0 = {s0.hi * up, s0.lo * up};
+        s1 = {s1.hi * up, s1.lo * up};
         if (df_less(tn, s0)) tn = s0;
         if (df_less(s1, tf)) tf = s1;
         if (!df_less(tn, tf) || !(tf.hi > 0.0f || (tf.hi == 0.0f && tf.lo > 0.0f))) {
@@ -508,399 +537,319 @@ __device__ void ray_begin(const KParams& kp, const TreeParams& tp, int64_t i, Ra
             return;
         }
     }
-    bool outside = tn.hi > 0.0f || (tn.hi == 0.0f && tn.lo > 0.0f);
-    if (SPHERE) R.rem = outside ? df_sub(tf, tn) : tf;
+    const bool outside = tn.hi > 0.0f || (tn.hi == 0.0f && tn.lo > 0.0f);
+    if (TRACE) R.t0 = outside ? DF{tn.hi * R.scale, tn.lo * R.scale} : DF{0.0f, 0.0f};
+    if (SPHERE) {
+        const DF rem = outside ? df_sub(tf, tn) : tf;
+        R.tend = rem.hi < 2.5f ? to_fixed(rem) : T_CAP;
+    }
+    const float grid = pow2i(tp.depth), cell = pow2i(-tp.depth);
+    const uint32_t qmax = (1u << tp.depth) - 1u;
+    R.t = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        R.p[a] = outside ? df_axpy(ou[a], tn, R.d[a], low_parts()[a * BLOCK]) : ou[a];
-        if (outside && R.d[a] != 0.0f && df_eq(near_a[a], tn)) R.p[a] = {R.d[a] > 0.0f ? 0.0f : 1.0f, 0.0f};
-        if (R.p[a].hi < 0.0f) R.p[a] = {0.0f, 0.0f};  // rounding guard
-        if (R.p[a].hi > 1.0f || (R.p[a].hi == 1.0f && R.p[a].lo > 0.0f)) R.p[a] = {1.0f, 0.0f};
+        DF p = m[a];
+        if (outside) p = df_eq(near_a[a], tn) ? DF{0.0f, 0.0f}  // the face it enters by
+                                              : df_axpy(p, tn, du[a].hi, du[a].lo);
+        if (p.hi < 0.0f) p = {0.0f, 0.0f};  // rounding guard
+        if (p.hi > 1.0f || (p.hi == 1.0f && p.lo > 0.0f)) p = {1.0f, 0.0f};
+        const uint32_t qa = quantize(p, grid, qmax);
+        const uint32_t k1 = qa + 1u;  // the next finest plane
+        R.q[a] = qa;
+        // position and direction, rounded down
+        const uint32_t o31 = (uint32_t)max(0, (int)__float2uint_rd(p.hi * 2147483648.0f) + __float2int_rd(p.lo * 2147483648.0f));
+        unsigned long long B = (unsigned long long)T_CAP, first = (unsigned long long)T_CAP;
+        uint32_t n = 1, d32 = 0;
+        if (rd[a].hi < FLAT) {
+            const uint32_t dh = __float2uint_rd(du[a].hi * 4294967296.0f);
+            const int dl = __float2int_rd(du[a].lo * 4294967296.0f);
+            d32 = dl < 0 && dh < (uint32_t)-dl ? 0u : dh + (uint32_t)dl;
+            const DF v = df_mul(df_from_plane((float)k1 * cell, p), rd[a].hi, rd[a].lo);
+            if (v.hi < 2.5f) first = (unsigned long long)max(0ll, to_fixed(v));
+            const float b = rd[a].hi * cell;
+            if (b < 2.5f) {
+                B = (unsigned long long)to_fixed(DF{b, rd[a].lo * cell});
+                n = __float2uint_rd(2.25f * grid * du[a].hi) + 1u;
+            }
+        }
+        axes().plane[a * BLOCK + threadIdx.x] = make_ulonglong2(first - (unsigned long long)k1 * B, B);
+        axes().pos[a * BLOCK + threadIdx.x] = make_uint2(o31, d32);
+        axes().kmax[a * BLOCK + threadIdx.x] = k1 + n;
     }
-    if (TRACE) R.t = outside ? tn : DF{0.0f, 0.0f};
-    const float scale = pow2i(tp.depth);
-    const uint32_t qmax = (1u << tp.depth) - 1u;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) R.q[a] = quantize(R.p[a], scale, qmax, R.d[a]);
     stack[0] = 0;
     R.node = 0;
     R.level = 0;
+    R.brick = 0;
     R.state = ST_DESCEND;
 }
 
-// Composites the current cell's entry over a segment of length `seg` (Eq.
-// 3-5): optical depth as a compensated sum, weight T_in (1 - e^{-sigma seg})
-// or the linear model's, SH emission of emitting leaves.  Returns true when
-// the ray is finished (T below t_stop) and its outputs are written.
-template <int K, int PREC>
-__device__ __forceinline__ bool composite(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R, float seg,
-                                          const float* sY) {
-    if (R.entry_x == ENTRY_EMPTY) return false;
-    float sigma = decode_sigma<PREC>(R.entry_y, tp.prec);
-    if (sigma < kp.sigma_min) sigma = 0.0f;
-    if (!(sigma > 0.0f)) return false;
-    // the emission first: its record loads are then in flight during the
-    // transmittance arithmetic (measured +1.5% with FP32 leaves)
-    const uint32_t rec = R.entry_x & ~LEAF_BIT;
-    float cr = 0.0f, cg = 0.0f, cb = 0.0f;
-    const bool emits = rec != NO_SH_RECORD;
-    if (emits) sh_emission<K, PREC>(tp, rec, R.entry_y, R.dirn, cr, cg, cb, sY);
+// Composites a segment of length `seg` with density sigma > 0 (Eq. 3-5):
+// optical depth as a compensated sum, weight w = T_in (1 - e^{-sigma seg}) or
+// the linear model's.
+__device__ __forceinline__ float composite(const KParams& kp, Ray& R, float sigma, float seg) {
     const float a = sigma * seg;
     const float Tin = R.T;
     const DF s = two_sum(R.od.hi, a);
     R.od = fast_two_sum(s.hi, __fadd_rn(s.lo, R.od.lo));
-    float w, Tout;
     if (kp.transmittance == PLO_TRANS_EXP) {
-        w = Tin * (-expm1f(-a));
-        Tout = expf(-(R.od.hi + R.od.lo));
-    } else {
-        Tout = fmaxf(0.0f, __fsub_rn(__fsub_rn(1.0f, R.od.hi), R.od.lo));
-        const float dT = fminf(Tin, a);
-        w = kp.transmittance == PLO_TRANS_LINEAR ? dT : 0.5f * dT * (Tin + Tout);
+        R.T = expf(-(R.od.hi + R.od.lo));
+        return Tin * (-expm1f(-a));
     }
-    if (emits || kp.activation != PLO_ACT_RELU) {
-        R.r = __fmaf_rn(w, act_fn(cr, kp.activation, kp.l_max), R.r);
-        R.g = __fmaf_rn(w, act_fn(cg, kp.activation, kp.l_max), R.g);
-        R.b = __fmaf_rn(w, act_fn(cb, kp.activation, kp.l_max), R.b);
-    }
-    R.T = Tout;
-    if (R.T < kp.t_stop || R.T <= 0.0f) {
-        ray_store(kp, i, R);
-        R.state = ST_IDLE;
-        return true;
-    }
-    return false;
+    R.T = fmaxf(0.0f, __fsub_rn(__fsub_rn(1.0f, R.od.hi), R.od.lo));
+    const float dT = fminf(Tin, a);
+    return kp.transmittance == PLO_TRANS_LINEAR ? dT : 0.5f * dT * (Tin + R.T);
 }
 
-// One cell: segment length, advance to the next cell, compositing.  Leaves
-// the lane in ST_DESCEND (next cell) or ST_IDLE (ray finished, outputs
-// written).
-template <int K, int PREC, bool TRACE, bool SPHERE>
-__device__ void leaf_step(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R, uint32_t* stack,
-                          const float* sY = nullptr) {
-    // segment: exit parameter of the current cell along each axis.  An FP32
-    // estimate (error below 6e-8 |1/d| + 2e-7 v) picks the candidate exit
-    // axes; only those get the double-float value.  Nearly always there is
-    // one candidate: its operands are picked by selects so that the
-    // double-float work is issued once per warp instead of once per axis.
-    const int L = R.level;
-    const int down = tp.depth - L;
-    const float size = pow2i(-L);
-    uint32_t c[3];
-    float planes[3], va[3], rh[3];
-    float vmin = INFINITY, rmin = 0.0f;
-    int ax = 0;  // axis of the smallest estimate
+// One cell: exit parameter, advance to the next cell, compositing (w: the
+// weight of the cell's emission).  Leaves the lane in ST_DESCEND (next cell),
+// in ST_LEAF (the next finest cell of the same brick, whose entry the caller
+// loads) or in ST_DONE / ST_DONE_LIMIT.
+//
+// The cell's three upper faces are finest-grid planes, so their parameters
+// are one 64-bit multiply-add each, and the segment is the difference of two
+// of them: exact to 2^-60, rounded once to FP32.  On the axes the ray does
+// not leave by, the next cell comes from the 31-bit position, which is
+// rounded down and at most 5 units low.  Where that hides a plane the ray has
+// just crossed, the next step finds the plane behind it and moves on with an
+// empty segment, so nothing is added to the wrong cell.
+template <bool TRACE, bool SPHERE, bool BRICKS>
+__device__ __forceinline__ void leaf_step(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R,
+                                          const uint32_t* stack, float sigma, float& w) {
+    const int down = tp.depth - R.level;
+    const uint32_t below = (1u << down) - 1u;
+    uint32_t k[3];
+    long long tk[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        rh[a] = low_parts()[(6 + a) * BLOCK];
-        c[a] = R.q[a] >> down;
-        planes[a] = (float)(c[a] + (R.d[a] > 0.0f ? 1u : 0u)) * size;
-        va[a] = INFINITY;
-        if (R.d[a] == 0.0f) continue;
-        va[a] = fmaxf(__fmul_rn(__fsub_rn(planes[a], R.p[a].hi), rh[a]), 0.0f);
-        if (va[a] < vmin) {
-            vmin = va[a];
-            rmin = fabsf(rh[a]);
-            ax = a;
-        }
+        k[a] = (R.q[a] | below) + 1u;
+        tk[a] = plane_at(a, k[a]);
     }
-    DF dt = {INFINITY, 0.0f};
-    DF dts[3];
-    bool cand[3];
-    int n_cand = 0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        dts[a] = {INFINITY, 0.0f};
-        cand[a] = va[a] <= vmin + 2.5e-7f * (fabsf(rh[a]) + rmin) + 1e-6f * vmin;
-        n_cand += cand[a] ? 1 : 0;
-    }
-    if (n_cand == 1) {
-        // the usual case: one candidate axis, gathered by selects so that the
-        // double-float work runs once for every lane whatever its axis
-        const float P = ax == 0 ? planes[0] : (ax == 1 ? planes[1] : planes[2]);
-        const DF pa = ax == 0 ? R.p[0] : (ax == 1 ? R.p[1] : R.p[2]);
-        const float rha = ax == 0 ? rh[0] : (ax == 1 ? rh[1] : rh[2]);
-        DF v = df_mul(df_from_plane(P, pa), rha, low_parts()[(3 + ax) * BLOCK]);
-        if (v.hi < 0.0f) v = {0.0f, 0.0f};
-        dt = v;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            if (a == ax) dts[a] = v;
-    } else {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!cand[a]) continue;
-            DF v = df_mul(df_from_plane(planes[a], R.p[a]), rh[a], low_parts()[(3 + a) * BLOCK]);
-            if (v.hi < 0.0f) v = {0.0f, 0.0f};
-            dts[a] = v;
-            if (df_less(v, dt)) dt = v;
-        }
-    }
+    long long te = min(tk[0], min(tk[1], tk[2]));
     bool last = false;  // the sphere proxy ends inside this cell
     if (SPHERE) {
-        if (df_less(dt, R.rem)) {
-            R.rem = df_sub(R.rem, dt);
-        } else {
-            dt = R.rem;
-            last = true;
-        }
+        last = R.tend <= te;
+        te = min(te, R.tend);
     }
-    const float seg = dt.hi;
+    te = max(te, R.t);
+    const unsigned long long dt = (unsigned long long)(te - R.t);
+    const float seg = __fmaf_rn((float)(uint32_t)(dt >> 32), 3.7252902984619140625e-9f,  // 2^(32 - T_FRAC)
+                                (float)(uint32_t)dt * 8.673617379884035472e-19f) *       // 2^-T_FRAC
+                      R.scale;
     ++R.steps;
-
     if (TRACE) {
-        int k = R.steps - 1;
-        DF t1 = two_sum(R.t.hi, dt.hi);
-        t1 = fast_two_sum(t1.hi, __fadd_rn(t1.lo, __fadd_rn(R.t.lo, dt.lo)));
-        if (k < kp.trace_max) {
-            size_t o = (size_t)i * kp.trace_max + k;
-            kp.tr_leaf[o] = R.entry_x == ENTRY_EMPTY ? -1
-                                                     : __ldg(tp.leaf_ids + (size_t)stack[(L - 1) * BLOCK] * 8 + R.slot);
-            kp.tr_t[2 * o] = R.t.hi;
-            kp.tr_t[2 * o + 1] = t1.hi;
+        auto param = [&](long long t) {  // caller's parameter, rounded once
+            const float h = (float)(uint32_t)(t >> 37) * R.scale;  // 24 bits: exact
+            const float l = (float)(t & ((1ll << 37) - 1)) * R.scale;
+            const DF s = two_sum(R.t0.hi, h * 1.1920928955078125e-7f);  // 2^(37 - T_FRAC)
+            return __fadd_rn(s.hi, __fadd_rn(__fadd_rn(s.lo, R.t0.lo), l * 8.673617379884035472e-19f));
+        };
+        const int c = R.steps - 1;
+        if (c < kp.trace_max) {
+            const size_t o = (size_t)i * kp.trace_max + c;
+            kp.tr_leaf[o] = R.entry_x == ENTRY_EMPTY
+                                ? -1
+                                : __ldg(tp.leaf_ids + (size_t)stack[(R.level - 1) * BLOCK] * 8 + child_slot(R, down));
+            kp.tr_t[2 * o] = param(R.t);
+            kp.tr_t[2 * o + 1] = param(te);
         }
-        R.t = t1;
     }
-
-    // advance to the exit point; snap the exit axes onto their planes.  Axes
-    // whose exit lies within 2^-36 (relative) of the first one count as exits
-    // too, so a ray through a shared edge or corner crosses it in one step
-    // instead of leaving a sliver segment behind.  The advance comes before
-    // the compositing, which does not depend on it: its double-float work
-    // then overlaps the wait for the SH record (measured on the depth-10
-    // luminaire: 379 -> 406 Mrays/s with FP32 leaves, 399 -> 436 with FP16;
-    // a finished ray drops the advanced position).
-    int l_anc = L;
-    const float tie = __fmaf_rn(dt.hi, 1.4551915228366852e-11f, dt.hi);
-    const float scale = pow2i(tp.depth);
-    const uint32_t qmax = (1u << tp.depth) - 1u;
-    bool left = false;
+    R.t = te;
+    const uint32_t t31 = (uint32_t)(te >> (T_FRAC - 31));
+    const int qs = 31 - tp.depth;
+    uint32_t diff = 0u;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (R.d[a] != 0.0f && (df_eq(dts[a], dt) || dts[a].hi <= tie)) {
-            R.p[a] = {planes[a], 0.0f};
-            const uint32_t cn = R.d[a] > 0.0f ? c[a] + 1u : c[a] - 1u;
-            left |= (cn >> L) != 0u;  // left the root cube (also catches 0 - 1)
-            // first (d > 0) or last (d < 0) finest cell of the neighbour
-            R.q[a] = R.d[a] > 0.0f ? cn << down : (c[a] << down) - 1u;
-            const int diff = 32 - __clz(cn ^ c[a]);
-            if (L - diff < l_anc) l_anc = L - diff;
-        } else {
-            R.p[a] = df_axpy(R.p[a], dt, R.d[a], low_parts()[a * BLOCK]);
-            R.q[a] = quantize(R.p[a], scale, qmax, R.d[a]);
+        const uint2 v = axes().pos[a * BLOCK + threadIdx.x];
+        uint32_t qn = (__umulhi(t31, v.y) + v.x) >> qs;
+        qn = min(max(qn, R.q[a]), k[a] - 1u);
+        if (TRACE) {  // the exact cell: no empty segments in the trace
+            if (qn + 1u < k[a] && plane_at(a, qn + 1u) <= te) ++qn;
         }
+        if (tk[a] <= te + T_TIE) qn = k[a];
+        diff |= qn ^ R.q[a];
+        R.q[a] = qn;
     }
+    const int msb = 31 - __clz(diff);  // the coarsest plane crossed
 
-    // composite the leaf (Eq. 3-5)
-    if (composite<K, PREC>(kp, tp, i, R, seg, sY)) return;
-    if (last) {
-        ray_store(kp, i, R);
-        R.state = ST_IDLE;
-        return;
+    R.state = ST_DONE;
+    if (sigma > 0.0f) {
+        w = composite(kp, R, sigma, seg);
+        if (R.T < kp.t_stop || R.T <= 0.0f) return;
     }
+    if (SPHERE && last) return;
     if (R.steps >= tp.max_steps) {
-        R.status = PLO_RAY_STEP_LIMIT;
         atomicOr(tp.flags, 1u);
-        ray_store(kp, i, R);
-        R.state = ST_IDLE;
+        R.state = ST_DONE_LIMIT;
         return;
     }
-    if (left) {
-        ray_store(kp, i, R);
-        R.state = ST_IDLE;
-        return;
+    if (msb >= tp.depth) return;  // left the cube
+    if (BRICKS) {
+        if (R.brick && msb < tp.brick_log) {
+            R.state = ST_LEAF;
+            return;
+        }
+        R.brick = 0;
     }
-    R.level = l_anc;
-    R.node = stack[l_anc * BLOCK];
+    // from the deepest common ancestor of this cell and the next
+    R.level = tp.depth - 1 - msb;
+    R.node = stack[R.level * BLOCK];
     R.state = ST_DESCEND;
 }
 
-// Leaves a brick across the face of axis `ax` at parameter tx (from the
-// brick entry point R.p): the exit point, snapped onto the planes it lies on
-// (the face, and any other axis whose next plane is crossed within 2^-36
-// of tx, so that a ray through an edge steps diagonally), its finest-grid
-// cell from the walk's own coordinates (no rounding: the walk counted every
-// plane crossed), then a descent from the deepest common ancestor of the
-// brick and that cell.
-__device__ __forceinline__ void brick_exit(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R,
-                                           uint32_t* stack, int ax, DF tx) {
-    const int s = tp.brick_log;
-    const uint32_t S = 1u << s;
-    const int Bl = tp.top_depth;
-    const float cell = pow2i(-tp.depth);
-    const float tie = __fmaf_rn(tx.hi, 1.4551915228366852e-11f, tx.hi);
-    bool left = false;
-    int l_anc = Bl;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const uint32_t base = R.q[a] & ~(S - 1u);  // the brick's corner on this axis
-        const uint32_t l = (R.loc >> (4 * a)) & 15u;
-        if (R.d[a] != 0.0f && (a == ax || R.tn[a].hi <= tie)) {
-            const bool up = R.d[a] > 0.0f;
-            const uint32_t qn = up ? base + l + 1u : base + l - 1u;  // wraps below 0: outside the cube
-            R.p[a] = {(float)(up ? qn : qn + 1u) * cell, 0.0f};
-            const uint32_t cb = base >> s, cn = qn >> s;
-            left |= (cn >> Bl) != 0u;
-            if (cn != cb) {
-                const int diff = 32 - __clz(cn ^ cb);
-                if (Bl - diff < l_anc) l_anc = Bl - diff;
-            }
-            R.q[a] = qn;
-        } else {
-            R.p[a] = df_axpy(R.p[a], tx, R.d[a], low_parts()[a * BLOCK]);
-            R.q[a] = base + l;
-        }
-    }
-    if (left || l_anc < 0) {
-        ray_store(kp, i, R);
-        R.state = ST_IDLE;
-        return;
-    }
-    R.level = l_anc;
-    R.node = stack[l_anc * BLOCK];
-    R.state = ST_DESCEND;
-}
+// Rays to walk, given out to the lanes of a warp.
+struct Claim {
+    int64_t next, end;  // warp-uniform range being handed out
+    bool more;          // the shared counter may have more
+};
 
-// One finest cell of a brick: the exit parameter is the smallest of the
-// three next-plane parameters (a digital differential analyser); composite
-// the cell over [tb, exit], then step one cell along the exit axis and load
-// that cell's entry for the next iteration.
-template <int K, int PREC, bool SPHERE>
-__device__ void brick_step(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R, uint32_t* stack,
-                           const float* sY = nullptr) {
-    int ax = 0;
-    DF tx = R.tn[0];
-    if (df_less(R.tn[1], tx)) {
-        ax = 1;
-        tx = R.tn[1];
-    }
-    if (df_less(R.tn[2], tx)) {
-        ax = 2;
-        tx = R.tn[2];
-    }
-    DF dt = df_sub(tx, R.tb);
-    if (dt.hi < 0.0f) dt = {0.0f, 0.0f};
-    bool last = false;  // the sphere proxy ends inside this cell
-    if (SPHERE) {
-        if (df_less(dt, R.rem)) {
-            R.rem = df_sub(R.rem, dt);
-        } else {
-            dt = R.rem;
-            last = true;
-        }
-    }
-    ++R.steps;
-    if (composite<K, PREC>(kp, tp, i, R, dt.hi, sY)) return;
-    if (last) {
-        ray_store(kp, i, R);
-        R.state = ST_IDLE;
-        return;
-    }
-    if (R.steps >= tp.max_steps) {
-        R.status = PLO_RAY_STEP_LIMIT;
-        atomicOr(tp.flags, 1u);
-        ray_store(kp, i, R);
-        R.state = ST_IDLE;
-        return;
-    }
-    // the next plane on the exit axis is one finest cell further: add
-    // 2^-D |1/d| (a power-of-two scaling of the double-float 1/d, exact)
-    const float sc = pow2i(-tp.depth);
-    const float rh = low_parts()[(6 + ax) * BLOCK], rl = low_parts()[(3 + ax) * BLOCK];
-    const DF step = rh > 0.0f ? DF{rh * sc, rl * sc} : DF{-rh * sc, -rl * sc};
-    const DF tnew = df_add(tx, step);
-    const bool up = ax == 0 ? R.d[0] > 0.0f : (ax == 1 ? R.d[1] > 0.0f : R.d[2] > 0.0f);
-    const int sh = 4 * ax;
-    const uint32_t l = (R.loc >> sh) & 15u;
-    if (up ? l + 1u < (1u << tp.brick_log) : l > 0u) {
-        R.tb = tx;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            if (a == ax) R.tn[a] = tnew;
-        R.loc = up ? R.loc + (1u << sh) : R.loc - (1u << sh);
-        const uint2 e = brick_entry(tp, R.node, R.loc);
-        R.entry_x = e.x;
-        R.entry_y = e.y;
-        return;
-    }
-    brick_exit(kp, tp, i, R, stack, ax, tx);
-}
-
-// The trace and sphere-proxy kernels keep more per-ray state, and degree-4
-// leaves (K = 25) a larger basis: 3 blocks per SM (80 registers) beats 4
-// with spills for them (measured; K = 25 on the depth-10 luminaire: 217 ->
-// 285 Mrays/s with FP32 leaves, 287 -> 326 with FP16).
+// Walks rays until none is left: the body of both render kernels.  One
+// iteration moves every lane that is at a cell past it, then descends every
+// lane towards its next cell.  tps: the tree (K > 0), or the batch's tree
+// table, its ray offsets and their number (K == 0).
+//
+// The emission of a leaf is not evaluated where the ray meets it: about 3 of
+// a warp's lanes do in an iteration (depth-9 luminaire), and their SH records
+// would be read and summed with the other lanes idle.  The lane puts record,
+// weight and itself into the warp's queue instead, and the warp evaluates the
+// queue when it holds up to 32 entries, one per lane, or when lanes take new
+// rays.  Every ray adds its own entries up in the order in which it met them,
+// so its result depends on nothing but itself.
 template <int K, int PREC, bool TRACE, bool SPHERE, bool BRICKS>
-__global__ void __launch_bounds__(BLOCK, (TRACE || SPHERE || K >= 25)
-                                              ? 3
-                                              : (BRICKS ? PLO_BRICK_MIN_BLOCKS : PLO_RENDER_MIN_BLOCKS))
-    k_render(KParams kp) {
-    // nodes of the top levels, staged once per (persistent) block, then the
-    // node id per level of the current cell's path (top_depth + 1 rows, one
-    // column per thread): dynamic shared memory sized by the tree, so that a
-    // shallow tree leaves more of the SM's memory to L1
-    extern __shared__ uint2 s_nodes[];
-    const TreeParams& tp = kp.tree;
-    for (int j = threadIdx.x; j < tp.n_top * 8; j += BLOCK) s_nodes[j] = tp.nodes[j];
-    __syncthreads();
-    uint32_t* stack = reinterpret_cast<uint32_t*>(s_nodes + tp.n_top * 8) + threadIdx.x;
-    __shared__ float s_Y[K * BLOCK];
-    float* sY = s_Y + threadIdx.x;
+__device__ __forceinline__ void walk_rays(const KParams& kp, const TreeParams* tps, const long long* offs, int n_trees,
+                                          const uint2* s_nodes, uint32_t* stack, Claim cl) {
+    __shared__ float4 s_queue[WARPS * 32];
+    __shared__ float s_dir[TRACE ? 1 : 3 * BLOCK];  // direction of each lane's ray, a column per lane
+    float* dir = s_dir + threadIdx.x;
+    float4* queue = s_queue + (threadIdx.x & ~31);
     const int lane = threadIdx.x & 31;
     const unsigned lanes_below = (1u << lane) - 1u;
-    const int64_t warp = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
-    int64_t next = 0, end = 0;  // warp-uniform range of rays being handed out
-    if (!kp.cursor) {
-        next = warp * kp.chunk;
-        if (next >= kp.n) return;  // whole warp exits together
-        end = min(next + kp.chunk, kp.n);
-    }
-    bool drained = false;
-
+    int queued = 0;         // entries of the warp's queue
+    unsigned mine = 0u;     // which of them are this lane's
     Ray R;
     R.state = ST_IDLE;
+    R.tree = 0;
     int64_t my = 0;
     for (;;) {
-        // idle lanes take the next rays; rays that miss the proxy finish at
-        // once, so repeat while lanes are idle and rays remain
-        for (;;) {
-            unsigned idle = __ballot_sync(0xffffffffu, R.state == ST_IDLE);
-            // refill in groups: ray setup runs with at least 4 lanes (or when
-            // no ray is left in flight; 4 measured faster than 8 and 16)
-            if (idle == 0u || (__popc(idle) < 4 && idle != 0xffffffffu)) break;
-            if (next >= end) {
-                if (!kp.cursor || drained) break;
-                unsigned long long b = 0;
-                if (lane == 0) b = atomicAdd(kp.cursor, (unsigned long long)RENDER_CLAIM);
-                b = __shfl_sync(0xffffffffu, b, 0);
-                if ((int64_t)b >= kp.n) {
-                    drained = true;
-                    break;
-                }
-                next = (int64_t)b;
-                end = min(next + RENDER_CLAIM, kp.n);
-            }
-            int64_t cand = next + __popc(idle & lanes_below);
-            next += __popc(idle);
-            if (R.state == ST_IDLE && cand < end) {
-                my = cand;
-                ray_begin<TRACE, SPHERE>(kp, tp, my, R, stack);
-                if (R.state != ST_IDLE) {
-                    float Y[K];
-                    sh_basis<K>(R.dirn[0], R.dirn[1], R.dirn[2], Y);
-#pragma unroll
-                    for (int k = 0; k < K; ++k) sY[k * BLOCK] = Y[k];
-                }
-            }
+        // what the lane's cell emits
+        float sigma = 0.0f;
+        if (R.state == ST_LEAF && R.entry_x != ENTRY_EMPTY) {
+            sigma = decode_sigma<PREC>(R.entry_y, K > 0 ? PREC : tps[R.tree].prec);
+            if (!(sigma >= kp.sigma_min)) sigma = 0.0f;
         }
-        const unsigned live = __ballot_sync(0xffffffffu, R.state != ST_IDLE);
-        if (live == 0u) break;
-        // every live lane is at a leaf, in a brick, or part-way down a
-        // descent longer than one step allows
-        if (BRICKS && R.state == ST_BRICK) brick_step<K, PREC, SPHERE>(kp, tp, my, R, stack, sY);
-        if (R.state == ST_LEAF) leaf_step<K, PREC, TRACE, SPHERE>(kp, tp, my, R, stack, sY);
+        const uint32_t rec = R.entry_x & ~LEAF_BIT;
+        const bool emits = !TRACE && sigma > 0.0f && (rec != NO_SH_RECORD || kp.activation != PLO_ACT_RELU);
+        const unsigned em = __ballot_sync(0xffffffffu, emits);
+        // lanes take new rays in groups: ray setup runs with at least
+        // REFILL of them, or when none is left in flight
+        const unsigned free = __ballot_sync(0xffffffffu, R.state <= ST_DONE_LIMIT);
+        const bool refill =
+            free == 0xffffffffu || (__popc(free) >= REFILL && (cl.more || cl.next < cl.end));
+        if (!TRACE && queued > 0 && (refill || queued + __popc(em) > 32)) {
+            __syncwarp();
+            if (lane < queued) {
+                const float4 e = queue[lane];
+                const uint32_t w = __float_as_uint(e.z);  // owner lane, scale exponent, tree
+                const uint32_t r = __float_as_uint(e.x);
+                const TreeParams& tp = K > 0 ? tps[0] : tps[w >> 16];
+                float c[3] = {0.0f, 0.0f, 0.0f};
+                if (r != NO_SH_RECORD) {
+                    sh_record<K, PREC>(tp, r, dir + (int)(w & 31u) - lane, c[0], c[1], c[2]);
+                    if (K > 0 ? PREC != PLO_PREC_FP32 : tp.prec != PLO_PREC_FP32) {
+                        const float sc = pow2i((int)((w >> 8) & 255u) - 127);
+                        c[0] *= sc;
+                        c[1] *= sc;
+                        c[2] *= sc;
+                    }
+                }
+                queue[lane] = make_float4(act_fn(c[0], kp.activation, kp.l_max), e.y,
+                                          act_fn(c[1], kp.activation, kp.l_max), act_fn(c[2], kp.activation, kp.l_max));
+            }
+            __syncwarp();
+            while (mine != 0u) {
+                const float4 e = queue[__ffs(mine) - 1];
+                mine &= mine - 1u;
+                R.r = __fmaf_rn(e.y, e.x, R.r);
+                R.g = __fmaf_rn(e.y, e.z, R.g);
+                R.b = __fmaf_rn(e.y, e.w, R.b);
+            }
+            __syncwarp();
+            queued = 0;
+        }
+        if (refill) {
+            if (R.state == ST_DONE || R.state == ST_DONE_LIMIT) {
+                ray_store(kp, my, R, R.state == ST_DONE ? PLO_RAY_OK : PLO_RAY_STEP_LIMIT);
+                R.state = ST_IDLE;
+            }
+            // rays that miss the proxy finish at once, so repeat while lanes
+            // are idle and rays remain
+            for (;;) {
+                const unsigned idle = __ballot_sync(0xffffffffu, R.state == ST_IDLE);
+                if (idle == 0u || (__popc(idle) < REFILL && idle != 0xffffffffu)) break;
+                if (cl.next >= cl.end) {
+                    if (!cl.more) break;
+                    unsigned long long b = 0;
+                    if (lane == 0) b = atomicAdd(kp.cursor, (unsigned long long)kp.claim);
+                    b = __shfl_sync(0xffffffffu, b, 0);
+                    if ((int64_t)b >= kp.n) {
+                        cl.more = false;
+                        break;
+                    }
+                    cl.next = (int64_t)b;
+                    cl.end = min(cl.next + kp.claim, kp.n);
+                }
+                const int64_t cand = cl.next + __popc(idle & lanes_below);
+                cl.next += __popc(idle);
+                if (R.state == ST_IDLE && cand < cl.end) {
+                    my = cand;
+                    if (K == 0) {
+                        int t = 0;
+                        while (t + 1 < n_trees && offs[t + 1] <= cand) ++t;
+                        R.tree = t;
+                    }
+                    ray_begin<TRACE, SPHERE>(kp, K > 0 ? tps[0] : tps[R.tree], my, R, stack, dir);
+                }
+            }
+            if (__ballot_sync(0xffffffffu, R.state != ST_IDLE) == 0u) break;
+        }
+        // every other lane is at a leaf, or part-way down a descent longer
+        // than one step allows
+        const TreeParams& tp = K > 0 ? tps[0] : tps[R.tree];
+        if (R.state == ST_LEAF) {
+            const int slot = queued + __popc(em & lanes_below);
+            float w = 0.0f;
+            leaf_step<TRACE, SPHERE, BRICKS>(kp, tp, my, R, stack, sigma, w);
+            if (emits) {
+                queue[slot] = make_float4(__uint_as_float(rec), w,
+                                          __uint_as_float((uint32_t)lane | (R.entry_y >> 24) << 8 | (uint32_t)R.tree << 16),
+                                          0.0f);
+                mine |= 1u << slot;
+            }
+            if (BRICKS && R.state == ST_LEAF) load_brick(tp, R);
+        }
+        queued += __popc(em);
         if (R.state == ST_DESCEND) descend_step<BRICKS, PREC>(tp, s_nodes, R, stack);
     }
+}
+
+// Resident blocks per SM: 4 (64 registers) hides the dependent node loads
+// best; the trace and sphere-proxy kernels keep more per-ray state and
+// degree-4 leaves (K = 25) a larger basis, and take 3 (80 registers).
+template <int K, int PREC, bool TRACE, bool SPHERE, bool BRICKS>
+__global__ void __launch_bounds__(BLOCK, TRACE || SPHERE || BRICKS || K >= 25 ? 3 : 4)
+    k_render(KParams kp) {
+    // the node id per level of the current cell's path (top_depth + 1 rows,
+    // one column per thread): dynamic shared memory sized by the tree, so
+    // that a shallow tree leaves more of the SM's memory to L1
+    extern __shared__ uint2 s_dyn[];
+    uint32_t* stack = reinterpret_cast<uint32_t*>(s_dyn) + threadIdx.x;
+    const int64_t warp = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
+    Claim cl = {0, 0, kp.cursor != nullptr};
+    if (!kp.cursor) {
+        cl.next = warp * kp.chunk;
+        if (cl.next >= kp.n) return;  // whole warp exits together
+        cl.end = min(cl.next + kp.chunk, kp.n);
+    }
+    walk_rays<K, PREC, TRACE, SPHERE, BRICKS>(kp, &kp.tree, nullptr, 1, nullptr, stack, cl);
 }
 
 // ---------------------------------------------------------------- batched render
@@ -913,17 +862,15 @@ constexpr int MAX_BATCH = 16;
 constexpr int BATCH_TOP_NODES = 73;  // levels 0..2 of a full octree
 
 struct BatchParams {
-    KParams base;  // render parameters and outputs (base.tree unused)
+    KParams base;  // render parameters, outputs, cursor (base.tree unused)
     TreeParams trees[MAX_BATCH];
     int64_t off[MAX_BATCH + 1];
     int32_t n_trees;
-    int32_t claim;
-    int32_t stack_off;           // entries (uint2) of staged nodes before the node stack
-    unsigned long long* cursor;  // zeroed before each launch
+    int32_t stack_off;  // entries (uint2) of staged nodes before the node stack
 };
 
 template <bool BRICKS>
-__global__ void __launch_bounds__(BLOCK, BRICKS ? PLO_BRICK_MIN_BLOCKS : PLO_RENDER_MIN_BLOCKS)
+__global__ void __launch_bounds__(BLOCK, 3)  // 4 blocks per SM spill: 4.6 against 3.4 ms (6 trees, 2.5M rays)
     k_render_batch(BatchParams bp) {
     extern __shared__ uint2 s_nodes[];
     __shared__ TreeParams s_tp[MAX_BATCH];
@@ -935,53 +882,10 @@ __global__ void __launch_bounds__(BLOCK, BRICKS ? PLO_BRICK_MIN_BLOCKS : PLO_REN
         for (int j = threadIdx.x; j < tp.n_top * 8; j += BLOCK) s_nodes[tp.s_off + j] = tp.nodes[j];
     }
     __syncthreads();
-    const KParams& kp = bp.base;
-    const long long total = s_off[bp.n_trees];
-    // per-thread node stack after the staged nodes (bp.stack_rows rows)
+    // per-thread node stack after the staged nodes
     uint32_t* stack = reinterpret_cast<uint32_t*>(s_nodes + bp.stack_off) + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    const unsigned lanes_below = (1u << lane) - 1u;
-
-    Ray R;
-    R.state = ST_IDLE;
-    R.tree = 0;
-    int64_t my = 0;
-    long long next = 0, end = 0;  // the warp's current claim (warp-uniform)
-    bool drained = false;
-    for (;;) {
-        for (;;) {
-            unsigned idle = __ballot_sync(0xffffffffu, R.state == ST_IDLE);
-            // refill in groups of at least 8 lanes
-            if (idle == 0u || (__popc(idle) < 8 && idle != 0xffffffffu)) break;
-            if (next >= end) {
-                if (drained) break;
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(bp.cursor, (unsigned long long)bp.claim);
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if ((long long)base >= total) {
-                    drained = true;
-                    break;
-                }
-                next = (long long)base;
-                end = min((long long)base + bp.claim, total);
-            }
-            const long long cand = next + __popc(idle & lanes_below);
-            next += __popc(idle);
-            if (R.state == ST_IDLE && cand < end) {
-                my = cand;
-                int t = 0;
-                while (t + 1 < bp.n_trees && s_off[t + 1] <= cand) ++t;
-                R.tree = t;
-                ray_begin<false, false>(kp, s_tp[t], my, R, stack);
-            }
-        }
-        const unsigned live = __ballot_sync(0xffffffffu, R.state != ST_IDLE);
-        if (live == 0u) break;
-        const TreeParams& tp = s_tp[R.tree];
-        if (BRICKS && R.state == ST_BRICK) brick_step<0, -1, false>(kp, tp, my, R, stack);
-        if (R.state == ST_LEAF) leaf_step<0, -1, false, false>(kp, tp, my, R, stack);
-        if (R.state == ST_DESCEND) descend_step<BRICKS, -1>(tp, s_nodes, R, stack);
-    }
+    walk_rays<0, -1, false, false, BRICKS>(bp.base, s_tp, s_off, bp.n_trees, s_nodes, stack,
+                                           Claim{0, 0, true});
 }
 
 // Point -> leaf lookup: descent from the root with the same tie rule.
@@ -1276,10 +1180,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
     kp.tr_leaf = tr_leaf;
     kp.tr_t = tr_t;
     kp.tr_count = tr_count;
-    // stage only the nodes of levels 0..2 (measured: the shared memory left
-    // over goes to L1, which serves the deeper node loads better)
-    if (kp.tree.n_top > BATCH_TOP_NODES) kp.tree.n_top = BATCH_TOP_NODES;
-    size_t smem = (size_t)kp.tree.n_top * 8 * sizeof(uint2) + (size_t)(kp.tree.top_depth + 1) * BLOCK * 4;
+    const size_t smem = (size_t)(kp.tree.top_depth + 1) * BLOCK * 4;
     cudaError_t e = cudaSuccess;
     cudaStream_t cs = (cudaStream_t)stream;
     unsigned long long* cursor = nullptr;
@@ -1295,6 +1196,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
             return cuda_error(e, "render work counter");
         }
         kp.cursor = cursor;
+        kp.claim = RENDER_CLAIM;
     }
     if (ordered) {
         // one scratch block: the claim counter, the (bin, block) table, the
@@ -1344,6 +1246,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
             return cuda_error(e, "render work counter and ray order");
         }
         kp.cursor = cursor;
+        kp.claim = RENDER_CLAIM;
     }
     const bool bricks = !TRACE && t->layout == PLO_LAYOUT_BRICKS;
     if (TRACE)
@@ -1538,7 +1441,7 @@ void apply_config(plo_batch* b) {
     for (int t = 0; t < b->n_trees; ++t) rows = std::max(rows, b->bp.trees[t].top_depth + 1);
     b->bp.stack_off = off;
     b->smem = (size_t)off * sizeof(uint2) + (size_t)rows * BLOCK * 4;
-    b->bp.claim = b->cfg.claim_rays;
+    b->bp.base.claim = b->cfg.claim_rays;
 }
 
 void (*batch_kernel(const plo_batch* b))(BatchParams) {
@@ -1626,7 +1529,7 @@ extern "C" plo_status plo_batch_create(const plo_tree* const* trees, int32_t n_t
         delete b;
         return cuda_error(e, "batch cursor allocation");
     }
-    b->bp.cursor = b->d_cursor;
+    b->bp.base.cursor = b->d_cursor;
     *out = b;
     return PLO_OK;
 }
