@@ -39,6 +39,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
@@ -930,6 +931,14 @@ __global__ void k_lookup(const uint2* nodes, const int32_t* leaf_ids, int depth,
     if (out_level) out_level[i] = lev;
 }
 
+// A small wavefront takes as long as its longest ray, and a warp's iteration
+// the longer the more lanes it moves, so its rays are spread over 16 warps
+// per SM before a warp takes 32 (1,021 rays of the depth-6 luminaire: 106 ->
+// 65 us, 16,384: 111 -> 101 us, of the depth-9 one: 292 -> 196 and 331 -> 279
+// us; over all the warps that fit, 16,384 rays take 129 and 352 us: the warps
+// then wait for each other's instructions).
+constexpr int SPREAD_WARPS = 16;
+
 // Persistent grid: as many blocks as fit on the device at once (occupancy
 // API), each warp owning a contiguous chunk of the rays.
 template <int K, int PREC, bool TRACE, bool SPHERE, bool BRICKS>
@@ -941,12 +950,10 @@ cudaError_t launch_k(KParams kp, int sm_count, size_t smem, cudaStream_t s) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, BLOCK, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    int64_t warps_needed = (kp.n + 31) / 32;
-    int64_t grid = (warps_needed + WARPS - 1) / WARPS;
-    int64_t max_grid = (int64_t)sm_count * per_sm;
-    if (grid > max_grid) grid = max_grid;
-    int64_t total_warps = grid * WARPS;
-    kp.chunk = (kp.n + total_warps - 1) / total_warps;
+    const int64_t max_warps = (int64_t)sm_count * per_sm * WARPS, few = (int64_t)sm_count * SPREAD_WARPS;
+    kp.chunk = std::max((kp.n + max_warps - 1) / max_warps, std::min<int64_t>((kp.n + few - 1) / few, 32));
+    const int64_t warps = std::min(max_warps, (kp.n + kp.chunk - 1) / kp.chunk);
+    const int64_t grid = (warps + WARPS - 1) / WARPS;
     fn<<<(unsigned)grid, BLOCK, smem, s>>>(kp);
     return cudaGetLastError();
 }
