@@ -984,10 +984,10 @@ cudaError_t launch_trunk_kernel(const gemm::TrunkMaps& maps, const gemm::TrunkAr
     const size_t smem = gemm::trunk_smem_bytes();
     cudaError_t e = cudaFuncSetAttribute(gemm::k_trunk<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int tiles = (a.M + gemm::BM - 1) / gemm::BM;
-    const int grid = tiles < sms ? tiles : sms;
-    if (grid < 1) return cudaSuccess;
-    gemm::k_trunk<BWD><<<grid, gemm::TR_THREADS, smem, s>>>(maps, a);
+    const int tiles = (a.M + 2 * gemm::BM - 1) / (2 * gemm::BM);
+    const int pairs = std::min(tiles, std::max(sms / 2, 1));
+    if (pairs < 1) return cudaSuccess;
+    gemm::k_trunk<BWD><<<2 * pairs, gemm::TR_THREADS, smem, s>>>(maps, a);
     return cudaGetLastError();
 }
 
@@ -997,7 +997,7 @@ cudaError_t launch_trunk(plo_mlp* m, int64_t samples, bool masks, bool keep, cud
     maps.x = m->mapA_H[0];
     gemm::TrunkArgs a{};
     for (int l = 0; l < DEPTH; ++l) {
-        maps.w[l] = m->mapW[l];
+        a.w[l] = m->W[l];
         maps.h[l] = m->mapA_H[l + 1];
         a.bias[l] = bias_ptr(m, m->master, l);
         a.bits[l] = masks ? m->HB[l + 1] : nullptr;
@@ -1016,7 +1016,7 @@ cudaError_t launch_trunk_bwd(plo_mlp* m, int64_t samples, cudaStream_t s) {
     gemm::TrunkArgs a{};
     for (int j = 0; j < DEPTH - 1; ++j) {
         const int l = DEPTH - 1 - j;
-        maps.w[j] = m->mapWT[l];
+        a.w[j] = m->WT[l];
         maps.h[j] = m->mapA_dZ[l - 1];
         a.bits[j] = m->HB[l];
     }
