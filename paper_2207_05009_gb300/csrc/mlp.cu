@@ -361,53 +361,90 @@ __device__ __forceinline__ uint32_t sigma24(float v) {
     return r >= 0xFF0000u ? 0xFEFFFFu : r;
 }
 
-// One distilled leaf per thread: the mean over its S jittered samples of
+// One distilled leaf per warp: the mean over its S jittered samples of
 // ReLU(sigma_raw) and of each raw SH coefficient, packed as plo_build_tree
 // packs a leaf: the record (FP32 coefficients, or 16-bit ones times a
 // power-of-two scale 2^e that puts the largest |coefficient| in [2^14, 2^15)
-// for FP16 and in [0.5, 1) for BF16) and the entry word.
+// for FP16 and in [0.5, 1) for BF16) and the entry word.  Lane l sums columns
+// 2l and 2l + 1 in sample order, so a sample's 256-byte row is one coalesced
+// load (524,288 samples, 8 per leaf: 128 us with a thread per leaf, which
+// loaded 4 bytes every 2 KB; now 20 us, 134 MB at 6.6 TB/s).
+constexpr int PACK_WARPS = 8;
 template <int PREC>
-__global__ void k_pack_leaves(const float* raw, int64_t nv, int S, int K, int stride, uint32_t* yword, uint8_t* emits,
-                              uint8_t* records) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nv) return;
-    float sig = 0.0f;
-    for (int s = 0; s < S; ++s) sig += fmaxf(__ldg(raw + (i * S + s) * OUT_PAD), 0.0f);
-    sig /= (float)S;
+__global__ void __launch_bounds__(32 * PACK_WARPS)
+    k_pack_leaves(const float* raw, int64_t nv, int S, int K, int stride, uint32_t* yword, uint8_t* emits,
+                  uint8_t* records) {
+    const int64_t i = (int64_t)blockIdx.x * PACK_WARPS + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (i >= nv) return;  // the whole warp leaves together
     const int nc = 3 * K;
-    uint8_t* rec = records + (size_t)i * stride;
-    // the means (written at once for FP32 records; for 16-bit ones this pass
-    // finds the largest |mean| and the next recomputes the same values)
+    const float2* row = reinterpret_cast<const float2*>(raw + i * S * OUT_PAD) + lane;
+    float c[2] = {0.0f, 0.0f};
+#pragma unroll 8
+    for (int s = 0; s < S; ++s) {
+        const float2 v = __ldg(row + (int64_t)s * (OUT_PAD / 2));
+        c[0] += lane == 0 ? fmaxf(v.x, 0.0f) : v.x;
+        c[1] += v.y;
+    }
     float m = 0.0f;
     bool any = false;
-    for (int k = 0; k < nc; ++k) {
-        float acc = 0.0f;
-        for (int s = 0; s < S; ++s) acc += __ldg(raw + (i * S + s) * OUT_PAD + 1 + k);
-        const float c = acc / (float)S;
-        any |= c != 0.0f;
-        m = fmaxf(m, fabsf(c));
-        if (PREC == PLO_PREC_FP32) reinterpret_cast<float*>(rec)[k] = c;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        c[u] /= (float)S;
+        const int k = 2 * lane + u - 1;
+        if (k >= 0 && k < nc) {
+            any |= c[u] != 0.0f;
+            m = fmaxf(m, fabsf(c[u]));
+        }
     }
-    emits[i] = any ? 1 : 0;
-    if (PREC == PLO_PREC_FP32) {
-        for (int b = 4 * nc; b < stride; ++b) rec[b] = 0;
-        yword[i] = __float_as_uint(sig);
-        return;
+    any = __any_sync(0xffffffffu, any);
+    uint8_t* rec = records + (size_t)i * stride;
+    if (lane == 0) emits[i] = any ? 1 : 0;
+    if constexpr (PREC == PLO_PREC_FP32) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int k = 2 * lane + u - 1;
+            if (k >= 0 && k < nc) reinterpret_cast<float*>(rec)[k] = c[u];
+        }
+        for (int b = 4 * nc + lane; b < stride; b += 32) rec[b] = 0;
+        if (lane == 0) yword[i] = __float_as_uint(c[0]);
+    } else {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        int e;
+        frexpf(m, &e);
+        if (PREC == PLO_PREC_FP16) e -= 15;
+        e = max(-126, min(127, e));
+        const float inv = ldexpf(1.0f, -e);
+        uint16_t* h = reinterpret_cast<uint16_t*>(rec);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int k = 2 * lane + u - 1;
+            const float v = c[u] * inv;
+            if (k >= 0 && k < nc)
+                h[k] = PREC == PLO_PREC_FP16 ? __half_as_ushort(__float2half_rn(v))
+                                             : __bfloat16_as_ushort(__float2bfloat16_rn(v));
+        }
+        for (int b = 2 * nc + lane; b < stride; b += 32) rec[b] = 0;
+        if (lane == 0) yword[i] = sigma24(c[0]) | (any ? (uint32_t)(e + 127) << 24 : 0u);
     }
-    int e;
-    frexpf(m, &e);
-    if (PREC == PLO_PREC_FP16) e -= 15;
-    e = max(-126, min(127, e));
-    const float inv = ldexpf(1.0f, -e);
-    uint16_t* h = reinterpret_cast<uint16_t*>(rec);
-    for (int k = 0; k < nc; ++k) {
-        float acc = 0.0f;
-        for (int s = 0; s < S; ++s) acc += __ldg(raw + (i * S + s) * OUT_PAD + 1 + k);
-        const float v = (acc / (float)S) * inv;
-        h[k] = PREC == PLO_PREC_FP16 ? __half_as_ushort(__float2half_rn(v)) : __bfloat16_as_ushort(__float2bfloat16_rn(v));
+}
+
+// Raw head outputs without their padding columns: out[row][0 .. n_out) =
+// raw[row][0 .. n_out), coalesced both ways, four elements a thread (200,001
+// rows of 196 bytes: 19 us; as a 2-D copy by the driver about 38 us).
+__global__ void __launch_bounds__(256) k_unpad_raw(const float* raw, int64_t n, int n_out, float* out) {
+    const int64_t total = n * n_out, base = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+    float v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int64_t i = base + 256 * j;
+        const int64_t row = total <= 0xFFFFFFFFll ? (int64_t)((uint32_t)i / (uint32_t)n_out) : i / n_out;
+        v[j] = i < total ? __ldg(raw + row * OUT_PAD + (i - row * n_out)) : 0.0f;
     }
-    for (int b = 2 * nc; b < stride; ++b) rec[b] = 0;
-    yword[i] = sigma24(sig) | (any ? (uint32_t)(e + 127) << 24 : 0u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (base + 256 * j < total) out[base + 256 * j] = v[j];
 }
 
 // Quadrature render of Eq. 3 from the head outputs, the loss of Eq. 7-9 and
@@ -979,15 +1016,15 @@ void padded_to_canonical(const plo_mlp* m, const std::vector<float>& p, float* c
 // 128-row tile stays in shared memory from the encoding to H[8]; the layers'
 // outputs H[1..8] are stored for the backward pass and the activation hook
 // (`keep` false: only H[8], which the head reads).
-template <bool BWD>
+template <bool BWD, bool BITS>
 cudaError_t launch_trunk_kernel(const gemm::TrunkMaps& maps, const gemm::TrunkArgs& a, int sms, cudaStream_t s) {
     const size_t smem = gemm::trunk_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(gemm::k_trunk<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(gemm::k_trunk<BWD, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int tiles = (a.M + 2 * gemm::BM - 1) / (2 * gemm::BM);
     const int pairs = std::min(tiles, std::max(sms / 2, 1));
     if (pairs < 1) return cudaSuccess;
-    gemm::k_trunk<BWD><<<2 * pairs, gemm::TR_THREADS, smem, s>>>(maps, a);
+    gemm::k_trunk<BWD, BITS><<<2 * pairs, gemm::TR_THREADS, smem, s>>>(maps, a);
     return cudaGetLastError();
 }
 
@@ -1005,7 +1042,8 @@ cudaError_t launch_trunk(plo_mlp* m, int64_t samples, bool masks, bool keep, cud
     a.store = keep ? 0xFFu : 0x80u;
     a.err = m->d_err;
     a.M = (int)samples;
-    return launch_trunk_kernel<false>(maps, a, m->sms, s);
+    return masks ? launch_trunk_kernel<false, true>(maps, a, m->sms, s)
+                 : launch_trunk_kernel<false, false>(maps, a, m->sms, s);
 }
 
 // The trunk's data-gradient chain (job j: layer l = 7 - j): dZ[l-1] =
@@ -1023,7 +1061,7 @@ cudaError_t launch_trunk_bwd(plo_mlp* m, int64_t samples, cudaStream_t s) {
     a.store = (1u << (DEPTH - 1)) - 1u;
     a.err = m->d_err;
     a.M = (int)samples;
-    return launch_trunk_kernel<true>(maps, a, m->sms, s);
+    return launch_trunk_kernel<true, true>(maps, a, m->sms, s);
 }
 
 plo_status forward_layers(plo_mlp* m, int64_t samples, cudaStream_t s, bool masks = false, bool keep = true) {
@@ -1340,8 +1378,8 @@ extern "C" plo_status plo_mlp_forward(plo_mlp* m, const float* d_points, int64_t
     k_pe_points<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d_points, n, m->H[0]);
     st = forward_layers(m, n, s);
     if (st != PLO_OK) return st;
-    cudaError_t e = cudaMemcpy2DAsync(d_raw, (size_t)m->n_out * 4, m->raw, OUT_PAD * 4, (size_t)m->n_out * 4, (size_t)n,
-                                      cudaMemcpyDeviceToDevice, s);
+    k_unpad_raw<<<(unsigned)((n * m->n_out + 1023) / 1024), 256, 0, s>>>(m->raw, n, m->n_out, d_raw);
+    const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PLO_OK : cuda_error(e, "raw output copy");
 }
 
@@ -1688,14 +1726,14 @@ plo_status distill(plo_mlp* m, int32_t depth, int32_t samples, float sigma_thres
                                                                           m->desc.seed, m->H[0]);
         st = forward_layers(m, nv * samples, s, false, false);
         if (st != PLO_OK) break;
-        const unsigned g = (unsigned)((nv + 127) / 128);
+        const unsigned g = (unsigned)((nv + PACK_WARPS - 1) / PACK_WARPS);
         uint8_t* rec = d_rec + (size_t)off * stride;
         if (precision == PLO_PREC_FP32)
-            k_pack_leaves<PLO_PREC_FP32><<<g, 128, 0, s>>>(m->raw, nv, samples, K, stride, d_yword + off, d_emits + off, rec);
+            k_pack_leaves<PLO_PREC_FP32><<<g, 32 * PACK_WARPS, 0, s>>>(m->raw, nv, samples, K, stride, d_yword + off, d_emits + off, rec);
         else if (precision == PLO_PREC_FP16)
-            k_pack_leaves<PLO_PREC_FP16><<<g, 128, 0, s>>>(m->raw, nv, samples, K, stride, d_yword + off, d_emits + off, rec);
+            k_pack_leaves<PLO_PREC_FP16><<<g, 32 * PACK_WARPS, 0, s>>>(m->raw, nv, samples, K, stride, d_yword + off, d_emits + off, rec);
         else
-            k_pack_leaves<PLO_PREC_BF16><<<g, 128, 0, s>>>(m->raw, nv, samples, K, stride, d_yword + off, d_emits + off, rec);
+            k_pack_leaves<PLO_PREC_BF16><<<g, 32 * PACK_WARPS, 0, s>>>(m->raw, nv, samples, K, stride, d_yword + off, d_emits + off, rec);
         e = cudaGetLastError();
     }
     if (st == PLO_OK && e == cudaSuccess) st = plo_mlp_check(m, stream);

@@ -76,7 +76,7 @@ struct TrunkMaps {
 struct TrunkArgs {
     const __nv_bfloat16* w[TR_LAYERS];  // B operand [256][K]: W_j (forward, K = 64 for j = 0), W_l^T (backward)
     const float* bias[TR_LAYERS];  // forward: layer j's bias
-    uint32_t* bits[TR_LAYERS];     // [M][8] words: forward, layer j's ReLU bits (written, nullable);
+    uint32_t* bits[TR_LAYERS];     // [M][8] words: forward, layer j's ReLU bits (written if BITS);
                                    // backward, the ReLU bits of H_l (read: the mask of the gradient)
     uint32_t store;                // bit j: store job j's output through h[j]
     unsigned int* err;          // bit 1: a pipeline wait gave up
@@ -176,8 +176,9 @@ __device__ __forceinline__ uint32_t interleave(uint32_t x) {
 
 // BWD: the data-gradient chain instead of the forward: per job
 // dZ_{l-1} = (dZ_l W_l) masked by the ReLU bits of H_l, l = 7 .. 1, starting
-// from the head's dZ_7 (four input K-blocks) with no bias.
-template <bool BWD>
+// from the head's dZ_7 (four input K-blocks) with no bias.  BITS (forward):
+// write the layers' ReLU bits, which only a training step needs.
+template <bool BWD, bool BITS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
     k_trunk(const __grid_constant__ TrunkMaps maps, TrunkArgs a) {
     constexpr uint32_t IDESC = sm100::idesc_bf16(2 * BM, TR_N, 0, 0);
@@ -385,7 +386,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                     }
                     load_mask(l + 1 < NJ ? r : r + 1, l + 1 < NJ ? l + 1 : 0, p);
                     const int row0 = (2 * tile + (int)rank) * BM;
-                    const bool bits = !BWD && a.bits[l];
+                    constexpr bool bits = !BWD && BITS;
                     if ((((a.store >> l) & 1u) || bits) && row0 < a.M) {
                         if ((a.store >> l) & 1u)
                             for (int kb = 0; kb < 4; ++kb)
@@ -450,12 +451,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                                 add2(x2, x3, b.z, b.w);
                                 packed[2 * j] = relu2(pack_bf16(x0, x1));
                                 packed[2 * j + 1] = relu2(pack_bf16(x2, x3));
-                                pos = (pos >> 1) | nonzero2(packed[2 * j]);
-                                pos = (pos >> 1) | nonzero2(packed[2 * j + 1]);
+                                if (BITS) {
+                                    pos = (pos >> 1) | nonzero2(packed[2 * j]);
+                                    pos = (pos >> 1) | nonzero2(packed[2 * j + 1]);
+                                }
                             }
-                            if (l == NJ - 1) pos = interleave(pos);  // the head's backward reads these in column order
-                            if (h == 0) pos0 = pos;
-                            else *bits = make_uint2(pos0, pos);
+                            if (BITS) {
+                                if (l == NJ - 1) pos = interleave(pos);  // the head's backward reads these in column order
+                                if (h == 0) pos0 = pos;
+                                else *bits = make_uint2(pos0, pos);
+                            }
                         }
                         uint8_t* blk = A + (size_t)(c >> 1) * TR_KBYTES + (size_t)rl * 128;
 #pragma unroll
