@@ -378,10 +378,30 @@ __host__ __device__ constexpr int wgrad_tmem_cols() {  // NIN accumulator column
     return NIN + 16 <= 32 ? 32 : (NIN + 16 <= 64 ? 64 : (NIN + 16 <= 128 ? 128 : (NIN + 16 <= 256 ? 256 : 512)));
 }
 
+//
+// A launch takes several layers (blockIdx.z): the split over the samples is
+// then a few thousand rows per CTA also for small batches, and the reduction,
+// 128 KB of atomics per CTA, is paid once per SM and wave instead of once per
+// layer (training step of 256 x 32 samples: 274 -> 135 us, 1024 x 64: 495 ->
+// 331 us, 4096 x 128: 2075 -> 1924 us; the layers' traffic is the floor of the
+// last, 4.3 GB at the copy rate of 6.7 TB/s).
+constexpr int WGRAD_JOBS = 9;
+struct WgradJobs {
+    CUtensorMap dZ[WGRAD_JOBS], H[WGRAD_JOBS];  // boxes of 64 x 64
+    float* dW[WGRAD_JOBS];
+    float* db[WGRAD_JOBS];  // nullable
+    int n_out[WGRAD_JOBS];
+};
+
 template <int NIN>
 __global__ void __launch_bounds__(THREADS, 1)
-    k_wgrad(const __grid_constant__ CUtensorMap tmDZ, const __grid_constant__ CUtensorMap tmH, float* dW, int n_out,
-            int M, int chunk, unsigned int* err, float* db) {
+    k_wgrad(const __grid_constant__ WgradJobs jobs, int M, int chunk, unsigned int* err) {
+    const CUtensorMap& tmDZ = jobs.dZ[blockIdx.z];
+    const CUtensorMap& tmH = jobs.H[blockIdx.z];
+    float* dW = jobs.dW[blockIdx.z];
+    float* db = jobs.db[blockIdx.z];
+    const int n_out = jobs.n_out[blockIdx.z];
+    if ((int)blockIdx.x * BM >= n_out) return;  // a layer with fewer outputs than the launch's widest
     constexpr int TMEM_COLS = wgrad_tmem_cols<NIN>();
     constexpr uint32_t IDESC = sm100::idesc_bf16(BM, NIN, 1, 1);
     constexpr uint32_t IDESC_ONES = sm100::idesc_bf16(BM, 16, 1, 0);

@@ -132,22 +132,38 @@ cudaError_t launch_gemm(const CUtensorMap& A, const CUtensorMap& B, const CUtens
     return cudaGetLastError();
 }
 
+// Weight gradients of the `n` layers of `jobs` (all with NIN inputs) over M
+// samples.  The samples are split so that the CTAs fill the SMs one to three
+// times over, more often only where a CTA still gets several thousand of
+// them: each adds its 128 x NIN sums with atomics.
 template <int NIN>
-cudaError_t launch_wgrad(const CUtensorMap& dZ, const CUtensorMap& H, float* dW, int n_out, int M, int sms,
-                         unsigned int* err, cudaStream_t s, float* db = nullptr) {
+cudaError_t launch_wgrad(const gemm::WgradJobs& jobs, int n, int M, int sms, unsigned int* err, cudaStream_t s) {
     const size_t smem = gemm::wgrad_smem_bytes<NIN>();
     cudaError_t e = cudaFuncSetAttribute(gemm::k_wgrad<NIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int out_tiles = (n_out + gemm::BM - 1) / gemm::BM;
-    int n_chunks = (2 * sms) / out_tiles;
+    int out_tiles = 0, tiles = 0;
+    for (int j = 0; j < n; ++j) {
+        const int t = (jobs.n_out[j] + gemm::BM - 1) / gemm::BM;
+        out_tiles = std::max(out_tiles, t);
+        tiles += t;
+    }
+    const int waves = std::min(3, std::max(1, M / 65536));
     const int blocks64 = M / 64;
-    if (n_chunks > blocks64) n_chunks = blocks64;
-    if (n_chunks < 1) n_chunks = 1;
+    int n_chunks = std::max(1, std::min(waves * sms / tiles, blocks64));
     const int chunk = ((blocks64 + n_chunks - 1) / n_chunks) * 64;
     n_chunks = (M + chunk - 1) / chunk;
-    dim3 grid(out_tiles, n_chunks);
-    gemm::k_wgrad<NIN><<<grid, gemm::THREADS, smem, s>>>(dZ, H, dW, n_out, M, chunk, err, db);
+    gemm::k_wgrad<NIN><<<dim3(out_tiles, n_chunks, n), gemm::THREADS, smem, s>>>(jobs, M, chunk, err);
     return cudaGetLastError();
+}
+
+void add_wgrad(gemm::WgradJobs& jobs, int& n, const CUtensorMap& dZ, const CUtensorMap& H, float* dW, int n_out,
+               float* db) {
+    jobs.dZ[n] = dZ;
+    jobs.H[n] = H;
+    jobs.dW[n] = dW;
+    jobs.db[n] = db;
+    jobs.n_out[n] = n_out;
+    ++n;
 }
 
 // ---------------------------------------------------------------- small kernels
@@ -1135,20 +1151,24 @@ plo_status backward_update(plo_mlp* m, int64_t M, cudaStream_t s) {
     gemm::EpiArgs ep{};
     ep.err = m->d_err;
     cudaError_t e;
+    gemm::WgradJobs wide{};  // the layers with 256 inputs: one launch at the end
+    int n_wide = 0;
     if (m->arch == PLO_ARCH_LINEAR_HEAD) {
-        e = launch_wgrad<WIDTH>(m->mapW_dO, m->mapW_H[DEPTH], m->grad + m->geom.off[DEPTH], OUT_PAD, (int)M, m->sms,
-                                m->d_err, s, bias_ptr(m, m->grad, DEPTH));
+        add_wgrad(wide, n_wide, m->mapW_dO, m->mapW_H[DEPTH], m->grad + m->geom.off[DEPTH], OUT_PAD,
+                  bias_ptr(m, m->grad, DEPTH));
         ep.out_bf16 = m->dZ[DEPTH - 1];
         ep.ldo = WIDTH;
         ep.bits = m->HB[DEPTH];
         ep.ldb = WIDTH / 32;
-        if (e == cudaSuccess)
-            e = launch_gemm<WIDTH, OUT_PAD>(m->mapA_dO, m->mapWT[DEPTH], &m->mapO_dZ7, ep, gemm::EPI_MASKBITS_BF16, (int)M, m->sms, s);
+        e = launch_gemm<WIDTH, OUT_PAD>(m->mapA_dO, m->mapWT[DEPTH], &m->mapO_dZ7, ep, gemm::EPI_MASKBITS_BF16, (int)M, m->sms, s);
     } else {
         const int SH = DEPTH + 1;
         // SH layer: dW = dO^T feat, db = column sums; d feat -> dZc[:, 0:128]
-        e = launch_wgrad<FEAT>(m->mapW_dO, m->mapW_H[SH], m->grad + m->geom.off[SH], OUT_PAD, (int)M, m->sms,
-                               m->d_err, s, bias_ptr(m, m->grad, SH));
+        gemm::WgradJobs narrow{};
+        int n_narrow = 0;
+        add_wgrad(narrow, n_narrow, m->mapW_dO, m->mapW_H[SH], m->grad + m->geom.off[SH], OUT_PAD,
+                  bias_ptr(m, m->grad, SH));
+        e = launch_wgrad<FEAT>(narrow, n_narrow, (int)M, m->sms, m->d_err, s);
         ep.out_bf16 = m->dZc;
         ep.ldo = COMB_PAD;
         ep.bits = m->HB[SH];
@@ -1156,9 +1176,8 @@ plo_status backward_update(plo_mlp* m, int64_t M, cudaStream_t s) {
         if (e == cudaSuccess)
             e = launch_gemm<FEAT, OUT_PAD>(m->mapA_dO, m->mapWT[SH], &m->mapO_dZc, ep, gemm::EPI_MASKBITS_BF16, (int)M, m->sms, s);
         // combined layer [features | sigma]: dW = dZc^T h8; d h8 -> dZ[7]
-        if (e == cudaSuccess)
-            e = launch_wgrad<WIDTH>(m->mapW_dZc, m->mapW_H[DEPTH], m->grad + m->geom.off[DEPTH], COMB_PAD, (int)M,
-                                    m->sms, m->d_err, s, bias_ptr(m, m->grad, DEPTH));
+        add_wgrad(wide, n_wide, m->mapW_dZc, m->mapW_H[DEPTH], m->grad + m->geom.off[DEPTH], COMB_PAD,
+                  bias_ptr(m, m->grad, DEPTH));
         ep.out_bf16 = m->dZ[DEPTH - 1];
         ep.ldo = WIDTH;
         ep.bits = m->HB[DEPTH];
@@ -1167,17 +1186,16 @@ plo_status backward_update(plo_mlp* m, int64_t M, cudaStream_t s) {
             e = launch_gemm<WIDTH, COMB_PAD>(m->mapA_dZc, m->mapWT[DEPTH], &m->mapO_dZ7, ep, gemm::EPI_MASKBITS_BF16, (int)M, m->sms, s);
     }
     // the trunk: the data gradients dZ[6] .. dZ[0] in one layer-fused chain
-    // from dZ[7], then every layer's weight gradient (each launch also sums
-    // the layer's bias gradient), reading dZ[l] and the layer's input H[l]
+    // from dZ[7], then the weight and bias gradients of every layer, reading
+    // dZ[l] and the layer's input H[l]
     if (e == cudaSuccess) e = launch_trunk_bwd(m, M, s);
-    for (int l = DEPTH - 1; l >= 0 && e == cudaSuccess; --l) {
-        if (l == 0)
-            e = launch_wgrad<PE_PAD>(m->mapW_dZ[0], m->mapW_H[0], m->grad + m->geom.off[0], WIDTH, (int)M, m->sms,
-                                     m->d_err, s, bias_ptr(m, m->grad, 0));
-        else
-            e = launch_wgrad<WIDTH>(m->mapW_dZ[l], m->mapW_H[l], m->grad + m->geom.off[l], WIDTH, (int)M, m->sms,
-                                    m->d_err, s, bias_ptr(m, m->grad, l));
-    }
+    for (int l = DEPTH - 1; l >= 1; --l)
+        add_wgrad(wide, n_wide, m->mapW_dZ[l], m->mapW_H[l], m->grad + m->geom.off[l], WIDTH, bias_ptr(m, m->grad, l));
+    if (e == cudaSuccess) e = launch_wgrad<WIDTH>(wide, n_wide, (int)M, m->sms, m->d_err, s);
+    gemm::WgradJobs first{};
+    int n_first = 0;
+    add_wgrad(first, n_first, m->mapW_dZ[0], m->mapW_H[0], m->grad + m->geom.off[0], WIDTH, bias_ptr(m, m->grad, 0));
+    if (e == cudaSuccess) e = launch_wgrad<PE_PAD>(first, n_first, (int)M, m->sms, m->d_err, s);
     if (e != cudaSuccess) return cuda_error(e, "MLP backward launch");
     // Adam with exponential decay lr0 -> lr1 over total_steps
     const double frac = std::fmin((double)(m->step - 1), (double)D.total_steps) / (double)D.total_steps;
@@ -1647,8 +1665,10 @@ extern "C" plo_status plo_wgrad_bf16(const void* d_dZ, int32_t n_out, const void
     if (st != PLO_OK) return st;
     const int sms = sm_count_of_current();
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = n_in == 256 ? launch_wgrad<256>(mZ, mH, d_dW, n_out, M, sms, d_err, s, d_db)
-                                : launch_wgrad<64>(mZ, mH, d_dW, n_out, M, sms, d_err, s, d_db);
+    gemm::WgradJobs job{};
+    int n = 0;
+    add_wgrad(job, n, mZ, mH, d_dW, n_out, d_db);
+    cudaError_t e = n_in == 256 ? launch_wgrad<256>(job, n, M, sms, d_err, s) : launch_wgrad<64>(job, n, M, sms, d_err, s);
     return e == cudaSuccess ? PLO_OK : cuda_error(e, "weight-gradient GEMM launch");
 }
 
