@@ -17,7 +17,8 @@
 // MMAs, the rest run the epilogue (warp w reads TMEM lanes 32*(w%4) .. +31).
 // k_gemm has two epilogue warpgroups (320 threads): the two warps of a lane
 // quadrant take half of the tile's 32-column chunks each, so every
-// sub-partition interleaves two epilogue warps; k_wgrad has one (192).  All mbarrier waits are bounded; a wait that gives up
+// sub-partition interleaves two epilogue warps; k_wgrad's two warpgroups hold
+// half of the tile's columns each, as running sums in registers.  All mbarrier waits are bounded; a wait that gives up
 // raises an abort flag in shared memory and a bit in the caller's error word,
 // every role then drains what it has in flight and the CTA frees its TMEM.
 #pragma once
@@ -32,7 +33,8 @@
 namespace plo {
 namespace gemm {
 
-constexpr int THREADS = 192;       // k_wgrad
+constexpr int WGRAD_EPI_GROUPS = 2;  // k_wgrad epilogue warpgroups
+constexpr int THREADS = 64 + 128 * WGRAD_EPI_GROUPS;  // k_wgrad
 constexpr int EPI_GROUPS = 2;      // k_gemm epilogue warpgroups
 constexpr int GEMM_THREADS = 64 + 128 * EPI_GROUPS;
 constexpr int BM = 128;
@@ -385,6 +387,14 @@ __host__ __device__ constexpr int wgrad_tmem_cols() {  // NIN accumulator column
 // layer (training step of 256 x 32 samples: 274 -> 135 us, 1024 x 64: 495 ->
 // 331 us, 4096 x 128: 2075 -> 1924 us; the layers' traffic is the floor of the
 // last, 4.3 GB at the copy rate of 6.7 TB/s).
+//
+// The tensor core truncates as it accumulates, so an error grows with the
+// length of a chain: every WGRAD_FLUSH k-blocks the accumulator goes to the
+// epilogue warps, which add it to their FP32 sums.  The operands of four
+// k-blocks take 6,000 cycles to arrive and their MMAs and the hand-over half
+// of that, so it costs no time (chains of 17,000 rows instead moved the
+// gradients by 7e-5, of the 3,456 rows that one launch per layer had by 1e-5).
+constexpr int WGRAD_FLUSH = 4;
 constexpr int WGRAD_JOBS = 9;
 struct WgradJobs {
     CUtensorMap dZ[WGRAD_JOBS], H[WGRAD_JOBS];  // boxes of 64 x 64
@@ -424,6 +434,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             sm100::mbar_init(&ctl->empty[s], 1);
         }
         sm100::mbar_init(&ctl->tfull[0], 1);
+        sm100::mbar_init(&ctl->tempty[0], 4 * WGRAD_EPI_GROUPS);
         sm100::mbar_init(&ctl->drain, 1);
         ctl->abort = 0;
         ctl->limit = sm100::WAIT_LIMIT;
@@ -474,6 +485,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         uint32_t ph = 0;
         bool ok = true, issued = false;
         for (int kb = 0; kb < n_kb; ++kb) {
+            const bool fresh = kb % WGRAD_FLUSH == 0;
+            if (fresh && kb > 0) {  // hand the accumulator over, and get it back
+                sm100::mma_commit(&ctl->tfull[0]);
+                if (!wait_or_abort(&ctl->tempty[0], (uint32_t)(kb / WGRAD_FLUSH - 1) & 1u, ctl, err)) {
+                    ok = false;
+                    break;
+                }
+            }
             if (!wait_or_abort(&ctl->full[stage], ph, ctl, err)) {
                 ok = false;
                 break;
@@ -485,10 +504,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int k = 0; k < 4; ++k) {
                 uint64_t adesc = sm100::smem_desc_sw128(a0 + 2048 * k, 8192, 1024);
                 uint64_t bdesc = sm100::smem_desc_sw128(b0 + 2048 * k, 8192, 1024);
-                sm100::mma_bf16(tmem, adesc, bdesc, IDESC, (kb | k) != 0);
+                sm100::mma_bf16(tmem, adesc, bdesc, IDESC, !fresh || k != 0);
                 if (db) {
                     uint64_t odesc = sm100::smem_desc_sw128(sm100::smem_addr(ones) + 32 * k, 16, 1024);
-                    sm100::mma_bf16(tmem + NIN, adesc, odesc, IDESC_ONES, (kb | k) != 0);
+                    sm100::mma_bf16(tmem + NIN, adesc, odesc, IDESC_ONES, !fresh || k != 0);
                 }
             }
             issued = true;
@@ -504,26 +523,41 @@ __global__ void __launch_bounds__(THREADS, 1)
             sm100::mbar_wait(&ctl->drain, 0);
         }
     } else if (warp >= 2 && n_kb > 0) {
-        const int q = warp & 3;
-        if (wait_or_abort(&ctl->tfull[0], 0, ctl, err)) {
-            sm100::tc_fence_after();
-            const int o = out_base + q * 32 + lane;
-#pragma unroll 1
-            for (int c = 0; c < NIN / 32; ++c) {
-                float v[32];
-                sm100::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
-                if (o < n_out) {
-                    float4* dst = reinterpret_cast<float4*>(dW + (size_t)o * NIN + c * 32);
+        constexpr int CHUNKS = NIN / 32 / WGRAD_EPI_GROUPS;  // 32-column chunks per warp
+        const int q = warp & 3, c0 = (warp - 2) / 4 * CHUNKS;
+        const bool sums = db && c0 == 0;
+        float acc[32 * CHUNKS], bias = 0.0f;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        atomicAdd(dst + j, make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
-                }
+        for (int j = 0; j < 32 * CHUNKS; ++j) acc[j] = 0.0f;
+        bool ok = true;
+        const int n_flush = (n_kb + WGRAD_FLUSH - 1) / WGRAD_FLUSH;
+        for (int f = 0; f < n_flush; ++f) {
+            ok = wait_or_abort(&ctl->tfull[0], (uint32_t)f & 1u, ctl, err);
+            if (!ok) break;
+            sm100::tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < CHUNKS; ++c) {
+                float v[32];
+                sm100::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((c0 + c) * 32), v);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) acc[32 * c + j] += v[j];
             }
-            if (db) {  // the 16 ones-columns all hold the row sum; the first one is used
+            if (sums) {  // the 16 ones-columns all hold the row sum; the first one is used
                 float v[32];
                 sm100::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)NIN, v);
-                if (o < n_out) atomicAdd(db + o, v[0]);
+                bias += v[0];
             }
+            sm100::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) sm100::mbar_arrive(&ctl->tempty[0]);
+        }
+        const int o = out_base + q * 32 + lane;
+        if (ok && o < n_out) {
+            float4* dst = reinterpret_cast<float4*>(dW + (size_t)o * NIN + c0 * 32);
+#pragma unroll
+            for (int j = 0; j < 8 * CHUNKS; ++j)
+                atomicAdd(dst + j, make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]));
+            if (sums) atomicAdd(db + o, bias);
         }
     }
     sm100::tc_fence_before();
