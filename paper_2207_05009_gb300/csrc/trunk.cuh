@@ -17,12 +17,13 @@
 // the biases and the ReLU bits: those used to be 4-byte accesses to global
 // memory in every epilogue.
 //
-// Measured on 524,288 rows (ncu, forward / data gradients): 645 / 495 us with
-// one CTA per tile, now 522 / 431 us; the stores of 2.15 / 1.88 GB alone take
-// 345 / 285 us at the rate the memory takes them, the MMAs alone 246 / 233 us
-// (everything but them taken out), everything but the stores 400 / 302 us.  So
-// the forward is bound by its epilogue, whose warps serve the two slots in
-// turn, and both by what the stores take from it.
+// Measured on 524,288 rows (ncu): the forward 645 us with one CTA per tile,
+// now 515 us with ReLU bits and all layers stored and 375 us with neither;
+// seven data-gradient layers 495 us, now eight in 445 us.  The stores of 2.15
+// GB alone take 345 us at the rate the memory takes them, the MMAs alone 246
+// us (everything but them taken out), everything but the stores 400 us.  So
+// it is bound by its epilogue, whose warps serve the two slots in turn, and by
+// what the stores take from it.
 //
 // Warp roles: 0 weight loads; 1 TMEM, MMA issue (lane 0 of the even CTA; the
 // odd one's passes "this K-block has landed here" on to the even CTA); 2 lane
@@ -65,16 +66,16 @@ __host__ __device__ constexpr size_t trunk_smem_bytes() {
     return 1024 + 2 * (size_t)TR_ABYTES + (size_t)TR_WSTAGES * TR_WBYTES + TR_BIAS_BYTES + 2 * TR_BITS_BYTES + 512;
 }
 
-// Indexed by job j of a tile: the forward's layer j (j = 0..7), or in the
-// backward chain the data gradient through layer l = 7 - j (j = 0..6).
+// Indexed by job j of a tile: the forward's layer j, or in the backward chain
+// the data gradient through layer 8 - j.
 struct TrunkMaps {
-    CUtensorMap x;                 // input tile, boxes 64 x 128, 128-byte swizzle: the encoded
-                                   // samples [M][64] (forward), d loss / d Z_7 [M][256] (backward)
+    CUtensorMap x;                 // input tile, boxes 64 x 128, 128-byte swizzle: the encoded samples [M][64]
+                                   // (forward), the gradient after the trunk [M][64 XKB] (backward)
     CUtensorMap h[TR_LAYERS];      // job j's output [M][256], boxes 64 x 128 (TMA stores)
 };
 
 struct TrunkArgs {
-    const __nv_bfloat16* w[TR_LAYERS];  // B operand [256][K]: W_j (forward, K = 64 for j = 0), W_l^T (backward)
+    const __nv_bfloat16* w[TR_LAYERS];  // B operand [256][K]: W_j (forward), W_l^T (backward); K = 64 XKB for j = 0
     const float* bias[TR_LAYERS];  // forward: layer j's bias
     uint32_t* bits[TR_LAYERS];     // [M][8] words: forward, layer j's ReLU bits (written if BITS);
                                    // backward, the ReLU bits of H_l (read: the mask of the gradient)
@@ -162,28 +163,17 @@ __device__ __forceinline__ uint32_t half_mask(uint32_t w) {
     asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(m) : "r"(w));
     return m;
 }
-// The same bits in column order.
-__device__ __forceinline__ uint32_t interleave(uint32_t x) {
-    uint32_t t = (x ^ (x >> 8)) & 0x0000FF00u;
-    x ^= t ^ (t << 8);
-    t = (x ^ (x >> 4)) & 0x00F000F0u;
-    x ^= t ^ (t << 4);
-    t = (x ^ (x >> 2)) & 0x0C0C0C0Cu;
-    x ^= t ^ (t << 2);
-    t = (x ^ (x >> 1)) & 0x22222222u;
-    return x ^ t ^ (t << 1);
-}
-
-// BWD: the data-gradient chain instead of the forward: per job
-// dZ_{l-1} = (dZ_l W_l) masked by the ReLU bits of H_l, l = 7 .. 1, starting
-// from the head's dZ_7 (four input K-blocks) with no bias.  BITS (forward):
-// write the layers' ReLU bits, which only a training step needs.
-template <bool BWD, bool BITS>
+// BWD: the data-gradient chain instead of the forward, with no bias: job 0
+// from the gradient of the layer after the trunk, then per job dZ_{l-1} =
+// (dZ_l W_l) masked by the ReLU bits of H_l.  (A GEMM of its own for job 0
+// took 90 us per 524,288 rows, and the chain read its 268 MB back.)  BITS
+// (forward): write the layers' ReLU bits, which only a training step needs.
+// XKB: K-blocks of the input tile.
+template <bool BWD, bool BITS, int XKB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
     k_trunk(const __grid_constant__ TrunkMaps maps, TrunkArgs a) {
     constexpr uint32_t IDESC = sm100::idesc_bf16(2 * BM, TR_N, 0, 0);
-    constexpr int NJ = BWD ? TR_LAYERS - 1 : TR_LAYERS;  // jobs per tile
-    constexpr int XKB = BWD ? 4 : 1;                      // K-blocks of the input tile
+    constexpr int NJ = TR_LAYERS;  // jobs per tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* act[2] = {smem, smem + TR_ABYTES};
@@ -238,7 +228,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
         const int c = lane & 7, r0 = lane >> 3;  // 16-byte chunk; rows r0, r0 + 4, ...
         for (int r = 0; ok && r < rounds; ++r)
             for (int l = 0; ok && l < NJ; ++l) {
-                const int nkb = (!BWD && l == 0) ? 1 : 4;
+                const int nkb = l == 0 ? XKB : 4;
                 const uint8_t* src = reinterpret_cast<const uint8_t*>(a.w[l]) +
                                      ((size_t)rank * TR_WROWS + r0) * (nkb * 128) + c * 16;
                 for (int kb = 0; kb < nkb; ++kb, w.next()) {
@@ -290,7 +280,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
         bool ok = true;
         for (int r = 0; ok && r < rounds; ++r)
             for (int l = 0; ok && l < NJ; ++l) {
-                const int nkb = (!BWD && l == 0) ? 1 : 4;
+                const int nkb = l == 0 ? XKB : 4;
                 for (int kb = 0; kb < nkb; ++kb, w.next()) {
                     if (!tr_wait(&ctl->wfull[w.s], w.ph, limit, ctl, a.err)) {
                         ok = false;
@@ -308,7 +298,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
         for (int r = 0; ok && r < rounds; ++r) {
             const int slots = tr_tile(r, 1, n_tiles) >= 0 ? 2 : 1;
             for (int l = 0; ok && l < NJ; ++l) {
-                const int nkb = (!BWD && l == 0) ? 1 : 4;
+                const int nkb = l == 0 ? XKB : 4;
                 TrStage v = w;
                 for (int p = 0; ok && p < slots; ++p) {
                     // the input: the loaded tile, or the previous layer's output
@@ -457,7 +447,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                                 }
                             }
                             if (BITS) {
-                                if (l == NJ - 1) pos = interleave(pos);  // the head's backward reads these in column order
                                 if (h == 0) pos0 = pos;
                                 else *bits = make_uint2(pos0, pos);
                             }
