@@ -6,16 +6,16 @@
 //   1. plo_trace_rays of the structure tree (the octree with zero leaves, so
 //      no ray saturates): per ray its cells in order with their canonical
 //      leaf ids and [t_in, t_out] -- the same walk as plo_render_rays;
-//   2. k_grad: per ray (one thread), the forward composite over the leaves
-//      with sigma = max(0, s) > 0 (Eq. 3-5), compacting them at the front of
-//      the ray's trace row as (leaf, delta) and (w, T_out); the loss (Sec.
-//      4.3, Eq. 7-9); then, back to front, d loss / d a_j and the SH
-//      gradients, added to the leaves with atomics;
+//   2. k_grad: per ray (one warp), the forward composite over the leaves
+//      with sigma = max(0, s) > 0 (Eq. 3-5), compacted at the front of the
+//      ray's trace row; the loss (Sec. 4.3, Eq. 7-9); then, back to front,
+//      d loss / d a_j and the SH gradients, added to the leaves with atomics;
 //   3. k_tv_terms, k_tv_grad: the TV terms and their gradients over the
 //      face-neighbour table and its reverse (two gathers, no atomics);
 //   4. k_adam: Adam over the raw densities and the coefficients.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -100,26 +100,45 @@ __device__ __forceinline__ void leaf_sigmoid(const float* kk, const float* Y, fl
     }
 }
 
-// One thread per ray.  Pass 1 composites the ray front to back over its
-// leaves (Eq. 3-5; the optical depth as a compensated sum, exponential
-// weights T_in (1 - e^{-a}), linear ones min(T_in, a)) and keeps, at the
-// front of the ray's trace row, each leaf with sigma > 0 as (leaf, delta)
-// and (w, T_out).  Pass 2 runs back to front over those entries with
-// g_j = sum_ch c_{j,ch} dL/dC_ch + dL/dalpha (dL/dw_j):
+// (hi + lo) + (bhi + blo) as an unevaluated sum of two floats
+__device__ __forceinline__ void df_add2(float& hi, float& lo, float bhi, float blo) {
+    const float s = __fadd_rn(hi, bhi), bb = __fsub_rn(s, hi);
+    const float e = __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(bhi, bb)), __fadd_rn(lo, blo));
+    hi = __fadd_rn(s, e);
+    lo = __fsub_rn(e, __fsub_rn(hi, s));
+}
+
+// One warp per ray, 32 of its leaves at a time.  The cells with a density are
+// first moved to the front of the ray's trace row.  Forward over them (Eq.
+// 3-5; the optical depth as a compensated sum, scanned over the lanes;
+// exponential weights T_in (1 - e^{-a}), linear ones min(T_in, a)), then the
+// loss, then backward with g_j = sum_ch c_{j,ch} dL/dC_ch + dL/dalpha (dL/dw_j):
 //   exponential: dL/da_j = T_out,j g_j - sum_{k>j} w_k g_k;
 //   linear:      dL/da_j = g_j before the leaf s where T reaches 0, minus
 //                g_s for j < s; 0 from s on;
 // d L / d s_j = dL/da_j delta_j (sigma_j > 0 here), and per channel
-// d L / d k_{j,ch,k} = w_j dL/dC_ch l_max sig (1 - sig) Y_k.
+// d L / d k_{j,ch,k} = w_j dL/dC_ch l_max sig (1 - sig) Y_k, the warp adding
+// one leaf's 3K values at a time, so that neighbouring ones share a sector.
+// With a thread per ray, which walked its leaves one after the other and
+// added every value to a sector of its own, 32,768 rays of the depth-7
+// luminaire (SH degree 2) took 192 us; now 54 us (step of 65,536
+// rays on the depth-8 luminaire, degree 3: 1326 -> 1046 us).
+constexpr int GRAD_WARPS = 4;
 template <int K>
-__global__ void __launch_bounds__(THREADS) k_grad(GradArgs p) {
-    const int64_t r = (int64_t)blockIdx.x * THREADS + threadIdx.x;
-    float loss = 0.0f;
-    if (r < p.n) {
+__global__ void __launch_bounds__(32 * GRAD_WARPS) k_grad(GradArgs p) {
+    constexpr unsigned ALL = 0xffffffffu;
+    constexpr int NV = (3 * K + 31) / 32;  // gradient values of a leaf per lane
+    __shared__ float s_loss[GRAD_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lanes_below = (1u << lane) - 1u;
+    const bool lin = p.transmittance == PLO_TRANS_LINEAR;
+    const float inv_l = 1.0f / p.l_max;
+    float loss_sum = 0.0f;
+    for (int64_t r = (int64_t)blockIdx.x * GRAD_WARPS + warp; r < p.n; r += (int64_t)gridDim.x * GRAD_WARPS) {
         int32_t cnt = p.tr_count[r];
         const bool over = cnt > p.max_cells;
         if (over) {
-            atomicOr(p.flags, 1u);
+            if (lane == 0) atomicOr(p.flags, 1u);
             cnt = 0;
         }
         float dw[3];
@@ -132,57 +151,83 @@ __global__ void __launch_bounds__(THREADS) k_grad(GradArgs p) {
         int64_t* row_leaf = p.tr_leaf + r * p.max_cells;
         int2* packed = reinterpret_cast<int2*>(row_leaf);
         float2* wt = reinterpret_cast<float2*>(p.tr_t + 2 * r * p.max_cells);
-        const bool lin = p.transmittance == PLO_TRANS_LINEAR;
 
-        // pass 1
-        float T = 1.0f, od_hi = 0.0f, od_lo = 0.0f, alpha = 0.0f;
-        float C[3] = {0.0f, 0.0f, 0.0f}, csat[3] = {0.0f, 0.0f, 0.0f};
-        int m = 0, sat = -1;
-        for (int j = 0; j < cnt; ++j) {
-            const int64_t leaf = row_leaf[j];
-            const float2 tt = wt[j];
-            if (leaf < 0) continue;
-            const float sv = __ldg(p.s + leaf);
-            if (!(sv > 0.0f)) continue;
-            const float delta = __fsub_rn(tt.y, tt.x);
-            const float a = sv * delta;
-            // compensated optical depth (two-sum)
-            const float sh = od_hi + a;
-            const float bb = sh - od_hi;
-            const float err = (od_hi - (sh - bb)) + (a - bb);
-            const float lo = od_lo + err;
-            od_hi = sh + lo;
-            od_lo = lo - (od_hi - sh);
-            float w, Tn;
-            if (!lin) {
-                w = T * (-expm1f(-a));
-                Tn = expf(-(od_hi + od_lo));
-            } else {
-                Tn = fmaxf(0.0f, __fsub_rn(__fsub_rn(1.0f, od_hi), od_lo));
-                w = fminf(T, a);
+        // cells with sigma = s > 0 to the front: (leaf, delta), (a, -)
+        int m = 0;
+        for (int base = 0; base < cnt; base += 32) {
+            const int j = base + lane;
+            const int64_t leaf = j < cnt ? row_leaf[j] : -1;
+            const float2 tt = j < cnt ? wt[j] : make_float2(0.0f, 0.0f);
+            const float sv = leaf >= 0 ? __ldg(p.s + leaf) : 0.0f;
+            const unsigned act = __ballot_sync(ALL, sv > 0.0f);
+            __syncwarp();
+            if (sv > 0.0f) {
+                const int at = m + __popc(act & lanes_below);
+                const float delta = __fsub_rn(tt.y, tt.x);
+                packed[at] = make_int2((int)leaf, __float_as_int(delta));
+                wt[at] = make_float2(sv * delta, 0.0f);
             }
-            float sg[3];
-            leaf_sigmoid<K>(p.k + leaf * 3 * K, Y, sg);
+            m += __popc(act);
+            __syncwarp();
+        }
+
+        // forward
+        float od_hi = 0.0f, od_lo = 0.0f, T_carry = 1.0f;
+        float C[3] = {0.0f, 0.0f, 0.0f}, alpha = 0.0f, csat[3] = {0.0f, 0.0f, 0.0f};
+        int sat = -1;
+        int64_t leaf = -1;  // of the last chunk, kept for the backward pass
+        float delta = 0.0f, w = 0.0f, Tn = 0.0f, sg[3] = {0.0f, 0.0f, 0.0f};
+        bool live = false;
+        int last = 0;
+        auto emission = [&]() {
+            if (live) leaf_sigmoid<K>(p.k + leaf * 3 * K, Y, sg);
+        };
+        for (int base = 0; base < m; base += 32) {
+            last = base;
+            const int j = base + lane;
+            const int2 e = j < m ? packed[j] : make_int2(-1, 0);
+            const float a = j < m ? wt[j].x : 0.0f;
+            leaf = e.x;
+            delta = __int_as_float(e.y);
+            float hi = a, lo = 0.0f;
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) C[ch] = __fmaf_rn(w, p.l_max * sg[ch], C[ch]);
-            alpha += w;
-            packed[m] = make_int2((int)leaf, __float_as_int(delta));
-            wt[m] = make_float2(w, Tn);
-            ++m;
-            T = Tn;
-            if (T <= 0.0f) {  // nothing behind contributes
+            for (int off = 1; off < 32; off <<= 1) {
+                const float uh = __shfl_up_sync(ALL, hi, off), ul = __shfl_up_sync(ALL, lo, off);
+                if (lane >= off) df_add2(hi, lo, uh, ul);
+            }
+            df_add2(hi, lo, od_hi, od_lo);
+            Tn = lin ? fmaxf(0.0f, __fsub_rn(__fsub_rn(1.0f, hi), lo)) : expf(-(hi + lo));
+            float T = __shfl_up_sync(ALL, Tn, 1);
+            if (lane == 0) T = T_carry;
+            live = j < m && T > 0.0f;  // nothing behind T = 0 contributes
+            w = !live ? 0.0f : (lin ? fminf(T, a) : T * (-expm1f(-a)));
+            emission();
+            if (live) {
+#pragma unroll
+                for (int ch = 0; ch < 3; ++ch) C[ch] = __fmaf_rn(w, p.l_max * sg[ch], C[ch]);
+                alpha += w;
+            }
+            if (j < m) wt[j] = make_float2(w, live ? Tn : -1.0f);
+            const unsigned stop = __ballot_sync(ALL, live && Tn <= 0.0f);
+            od_hi = __shfl_sync(ALL, hi, 31);
+            od_lo = __shfl_sync(ALL, lo, 31);
+            T_carry = __shfl_sync(ALL, Tn, 31);
+            if (stop) {
+                const int at = __ffs(stop) - 1;
                 if (lin) {
-                    sat = m - 1;
+                    sat = base + at;
 #pragma unroll
-                    for (int ch = 0; ch < 3; ++ch) csat[ch] = p.l_max * sg[ch];
+                    for (int ch = 0; ch < 3; ++ch) csat[ch] = p.l_max * __shfl_sync(ALL, sg[ch], at);
                 }
                 break;
             }
         }
+        alpha = warp_sum(alpha);
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) C[ch] = warp_sum(C[ch]);
 
         // the loss on values divided by l_max (denominator held constant)
-        float dC[3];
-        const float inv_l = 1.0f / p.l_max;
+        float loss = 0.0f, dC[3];
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) {
             const float cn = C[ch] * inv_l, gn = __ldg(p.rgb_gt + 3 * r + ch) * inv_l;
@@ -198,65 +243,81 @@ __global__ void __launch_bounds__(THREADS) k_grad(GradArgs p) {
             dA = 2.0f * da * p.inv_n;
         }
         if (over) loss = 0.0f;
-        if (p.ray_out) {
-            float* o = p.ray_out + 5 * r;
-            const float nan = __int_as_float(0x7fc00000);
-            o[0] = over ? nan : C[0];
-            o[1] = over ? nan : C[1];
-            o[2] = over ? nan : C[2];
-            o[3] = over ? nan : alpha;
-            o[4] = over ? nan : loss;
+        loss_sum += loss;
+        if (p.ray_out && lane < 5) {
+            const float v = lane == 0 ? C[0] : lane == 1 ? C[1] : lane == 2 ? C[2] : lane == 3 ? alpha : loss;
+            p.ray_out[5 * r + lane] = over ? __int_as_float(0x7fc00000) : v;
         }
 
-        // pass 2, back to front
+        // backward
         const float gsat = sat >= 0 ? __fmaf_rn(csat[0], dC[0], __fmaf_rn(csat[1], dC[1], __fmaf_rn(csat[2], dC[2], dA)))
                                     : 0.0f;
-        float after = 0.0f;  // sum over the later leaves of w g
-        for (int j = m - 1; j >= 0; --j) {
-            const int2 e = packed[j];
-            const float2 q = wt[j];
-            const int64_t leaf = e.x;
-            const float delta = __int_as_float(e.y), w = q.x, Tn = q.y;
-            float sg[3];
-            leaf_sigmoid<K>(p.k + leaf * 3 * K, Y, sg);
+        float yv[NV];  // this lane's basis values among a leaf's 3K gradients
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            yv[i] = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 3 * K; ++q)
+                if (q == lane + 32 * i) yv[i] = Y[q % K];
+        }
+        float after = 0.0f;  // sum over the later chunks' leaves of w g
+        for (int base = last; base >= 0 && m > 0; base -= 32) {
+            const int j = base + lane;
+            if (base != last) {
+                __syncwarp();
+                const int2 e = packed[j];
+                const float2 q = wt[j];
+                leaf = e.x;
+                delta = __int_as_float(e.y);
+                w = q.x;
+                Tn = q.y;
+                live = true;  // a stop ends the last chunk
+                emission();
+            }
             float g = dA;
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) g = __fmaf_rn(p.l_max * sg[ch], dC[ch], g);
             float da;
             if (!lin) {
-                da = __fmaf_rn(Tn, g, -after);
-                after = __fmaf_rn(w, g, after);
+                const float wg = live ? w * g : 0.0f;
+                float suf = wg;  // over this lane and the later ones
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const float v = __shfl_down_sync(ALL, suf, off);
+                    if (lane + off < 32) suf += v;
+                }
+                const float later = __shfl_down_sync(ALL, suf, 1);
+                da = __fmaf_rn(Tn, g, -((lane < 31 ? later : 0.0f) + after));
+                after += __shfl_sync(ALL, suf, 0);
             } else {
                 da = sat < 0 ? g : (j < sat ? g - gsat : 0.0f);
             }
-            atomicAdd(p.gs + leaf, da * delta);
-            float* gk = p.gk + leaf * 3 * K;
+            if (live) atomicAdd(p.gs + leaf, da * delta);
             float dz[3];
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) dz[ch] = w * dC[ch] * p.l_max * sg[ch] * (1.0f - sg[ch]);
-            if constexpr ((3 * K) % 4 == 0) {
-                // a leaf's 3K coefficients are whole 16-byte groups (rows of
-                // 3K floats from a 256-byte aligned base): one vector
-                // reduction per four coefficients instead of four
+            for (unsigned todo = __ballot_sync(ALL, live); todo; todo &= todo - 1u) {
+                const int src = __ffs(todo) - 1;
+                const int64_t lf = __shfl_sync(ALL, (int)leaf, src);
+                const float d0 = __shfl_sync(ALL, dz[0], src), d1 = __shfl_sync(ALL, dz[1], src);
+                const float d2 = __shfl_sync(ALL, dz[2], src);
+                float* gk = p.gk + lf * 3 * K;
 #pragma unroll
-                for (int q = 0; q < 3 * K / 4; ++q) {
-                    float4 v;
-                    v.x = dz[(4 * q + 0) / K] * Y[(4 * q + 0) % K];
-                    v.y = dz[(4 * q + 1) / K] * Y[(4 * q + 1) % K];
-                    v.z = dz[(4 * q + 2) / K] * Y[(4 * q + 2) % K];
-                    v.w = dz[(4 * q + 3) / K] * Y[(4 * q + 3) % K];
-                    atomicAdd(reinterpret_cast<float4*>(gk) + q, v);
+                for (int i = 0; i < NV; ++i) {
+                    const int q = lane + 32 * i;
+                    if (q < 3 * K) atomicAdd(gk + q, (q < K ? d0 : q < 2 * K ? d1 : d2) * yv[i]);
                 }
-            } else {
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch)
-#pragma unroll
-                    for (int kk = 0; kk < K; ++kk) atomicAdd(gk + ch * K + kk, dz[ch] * Y[kk]);
             }
         }
+        __syncwarp();
     }
-    loss = warp_sum(loss);
-    if ((threadIdx.x & 31) == 0 && loss != 0.0f) atomicAdd(p.acc, loss * p.inv_n);
+    if (lane == 0) s_loss[warp] = loss_sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.0f;
+        for (int i = 0; i < GRAD_WARPS; ++i) t += s_loss[i];
+        if (t != 0.0f) atomicAdd(p.acc, t * p.inv_n);
+    }
 }
 
 // TV of C channels x [n][C], pass 1, over every (leaf i, channel c) in a
@@ -337,7 +398,8 @@ unsigned grid_of(int64_t n, int threads) { return (unsigned)((n + threads - 1) /
 
 template <int K>
 cudaError_t launch_grad(const GradArgs& a, cudaStream_t s) {
-    k_grad<K><<<grid_of(a.n, THREADS), THREADS, 0, s>>>(a);
+    const unsigned blocks = std::min<unsigned>(grid_of(a.n, GRAD_WARPS), 12u * 152u);
+    k_grad<K><<<blocks, 32 * GRAD_WARPS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
