@@ -372,7 +372,7 @@ __device__ __forceinline__ uint32_t child_slot(const Ray& R, int sh) {
 // descent among its lanes, 5.7 levels (depth-10 luminaire, 16M room rays):
 // 4 levels per step measured 348 -> 365 Mrays/s with FP32 leaves, 390 ->
 // 397 with FP16; 2 levels gained nothing and 1 level lost.
-template <bool BRICKS, int PREC>
+template <bool BRICKS>
 __device__ __forceinline__ void descend_step(const TreeParams& tp, const uint2* s_nodes, Ray& R, uint32_t* stack) {
     // the child bits of the levels to come, at the top of a word per axis
     uint32_t x[3];
@@ -399,20 +399,6 @@ __device__ __forceinline__ void descend_step(const TreeParams& tp, const uint2* 
             if (!(e.x & LEAF_BIT)) e = make_uint2(ENTRY_EMPTY, 0u);
             R.entry_x = e.x;
             R.entry_y = e.y;
-            // the SH record is read in the next iteration: start pulling it
-            // into L2 now, for 16-bit records (measured on the depth-10
-            // workload: FP16 427 -> 436 Mrays/s with it, FP32 410 -> 404,
-            // so FP32 records are left to the load itself; before the leaf
-            // step advanced ahead of its compositing FP32 gained, 366 ->
-            // 379).  The choice is made at compile time: as a run-time test
-            // it cost the FP16 kernel 9%.
-            const uint32_t rec = e.x & ~LEAF_BIT;
-            constexpr bool always = PREC > 0, never = PREC == PLO_PREC_FP32;
-            if (!never && (always || tp.prec != PLO_PREC_FP32) && e.x != ENTRY_EMPTY && rec != NO_SH_RECORD) {
-                const char* a = reinterpret_cast<const char*>(tp.sh) + (size_t)rec * tp.sh_stride;
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(a + tp.sh_stride - 1));
-            }
             return;
         }
         stack[R.level * BLOCK] = e.x;
@@ -714,7 +700,10 @@ struct Claim {
 // weight and itself into the warp's queue instead, and the warp evaluates the
 // queue when it holds up to 32 entries, one per lane, or when lanes take new
 // rays.  Every ray adds its own entries up in the order in which it met them,
-// so its result depends on nothing but itself.
+// so its result depends on nothing but itself.  (Pulling 16-bit records into
+// L2 when the descent finds them, which helped while they were read one
+// iteration later, now costs 3%: 9M rays, depth 9, FP16 12.48 -> 12.10 ms
+// without it; FP32 records at the time they are queued: +2%.)
 template <int K, int PREC, bool TRACE, bool SPHERE, bool BRICKS>
 __device__ __forceinline__ void walk_rays(const KParams& kp, const TreeParams* tps, const long long* offs, int n_trees,
                                           const uint2* s_nodes, uint32_t* stack, Claim cl) {
@@ -828,7 +817,7 @@ __device__ __forceinline__ void walk_rays(const KParams& kp, const TreeParams* t
             if (BRICKS && R.state == ST_LEAF) load_brick(tp, R);
         }
         queued += __popc(em);
-        if (R.state == ST_DESCEND) descend_step<BRICKS, PREC>(tp, s_nodes, R, stack);
+        if (R.state == ST_DESCEND) descend_step<BRICKS>(tp, s_nodes, R, stack);
     }
 }
 
