@@ -243,9 +243,11 @@ plo_status plo_render_rays_host_noalloc(const plo_tree* tree, const float* h_ray
 typedef struct plo_batch plo_batch;
 
 /* Launch shape of the batch kernel.
- *   claim_rays     rays a warp takes from the queue at a time (multiple of 32)
+ *   claim_rays     rays a warp takes from the queue at a time (multiple of 32;
+ *                  an upper bound: small batches are handed out in smaller parts)
  *   blocks_per_sm  resident blocks per SM (0: as many as fit)
- *   top_nodes      nodes per tree staged in shared memory (0..73) */
+ *   top_nodes      0..73, kept and reported but without effect: the kernel reads
+ *                  all nodes through L1, which measured faster than staging them */
 typedef struct {
     int32_t claim_rays;
     int32_t blocks_per_sm;

@@ -71,8 +71,6 @@ struct TreeParams {
     int32_t top_depth;    // level of the brick cells (= depth for the octree layout)
     int32_t sh_stride;
     int32_t depth;
-    int32_t n_top;   // nodes staged in shared memory (ids 0 .. n_top-1)
-    int32_t s_off;   // their offset in the block's shared node table (entries)
     int32_t K, prec;
     int32_t max_steps;
     float bmin[3], inv_ext[3], inv_ext_lo[3];  // 1/extent as a double-float
@@ -339,11 +337,6 @@ __device__ __forceinline__ long long to_fixed(DF v) {
     return __float2ll_rn(v.hi * s) + __float2ll_rn(v.lo * s);
 }
 
-__device__ __forceinline__ uint2 load_entry(const TreeParams& tp, const uint2* s_nodes, uint32_t node, uint32_t slot) {
-    if (s_nodes && node < (uint32_t)tp.n_top) return s_nodes[tp.s_off + node * 8 + slot];
-    return __ldg(tp.nodes + (size_t)node * 8 + slot);
-}
-
 // Entry of the finest cell R.q of a brick: index = Morton interleave of the
 // brick-local coordinates (mirrored back), x lowest.
 __device__ __forceinline__ uint32_t spread3(uint32_t x) { return (x & 1u) | ((x & 2u) << 2) | ((x & 4u) << 4); }
@@ -373,7 +366,7 @@ __device__ __forceinline__ uint32_t child_slot(const Ray& R, int sh) {
 // 4 levels per step measured 348 -> 365 Mrays/s with FP32 leaves, 390 ->
 // 397 with FP16; 2 levels gained nothing and 1 level lost.
 template <bool BRICKS>
-__device__ __forceinline__ void descend_step(const TreeParams& tp, const uint2* s_nodes, Ray& R, uint32_t* stack) {
+__device__ __forceinline__ void descend_step(const TreeParams& tp, Ray& R, uint32_t* stack) {
     // the child bits of the levels to come, at the top of a word per axis
     uint32_t x[3];
 #pragma unroll
@@ -385,7 +378,7 @@ __device__ __forceinline__ void descend_step(const TreeParams& tp, const uint2* 
         slot = __funnelshift_l(x[0], slot, 1);
 #pragma unroll
         for (int a = 0; a < 3; ++a) x[a] <<= 1;
-        uint2 e = load_entry(tp, s_nodes, R.node, slot);
+        uint2 e = __ldg(tp.nodes + (size_t)R.node * 8 + slot);
         ++R.level;
         if ((e.x & LEAF_BIT) || R.level >= tp.top_depth) {  // leaf, empty octant, brick (or a malformed table)
             R.state = ST_LEAF;
@@ -706,7 +699,7 @@ struct Claim {
 // without it; FP32 records at the time they are queued: +2%.)
 template <int K, int PREC, bool TRACE, bool SPHERE, bool BRICKS>
 __device__ __forceinline__ void walk_rays(const KParams& kp, const TreeParams* tps, const long long* offs, int n_trees,
-                                          const uint2* s_nodes, uint32_t* stack, Claim cl) {
+                                          uint32_t* stack, Claim cl) {
     __shared__ float4 s_queue[WARPS * 32];
     __shared__ float s_dir[TRACE ? 1 : 3 * BLOCK];  // direction of each lane's ray, a column per lane
     float* dir = s_dir + threadIdx.x;
@@ -817,7 +810,7 @@ __device__ __forceinline__ void walk_rays(const KParams& kp, const TreeParams* t
             if (BRICKS && R.state == ST_LEAF) load_brick(tp, R);
         }
         queued += __popc(em);
-        if (R.state == ST_DESCEND) descend_step<BRICKS>(tp, s_nodes, R, stack);
+        if (R.state == ST_DESCEND) descend_step<BRICKS>(tp, R, stack);
     }
 }
 
@@ -830,8 +823,8 @@ __global__ void __launch_bounds__(BLOCK, TRACE || SPHERE || BRICKS || K >= 25 ? 
     // the node id per level of the current cell's path (top_depth + 1 rows,
     // one column per thread): dynamic shared memory sized by the tree, so
     // that a shallow tree leaves more of the SM's memory to L1
-    extern __shared__ uint2 s_dyn[];
-    uint32_t* stack = reinterpret_cast<uint32_t*>(s_dyn) + threadIdx.x;
+    extern __shared__ uint32_t s_stack[];
+    uint32_t* stack = s_stack + threadIdx.x;
     const int64_t warp = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
     Claim cl = {0, 0, kp.cursor != nullptr};
     if (!kp.cursor) {
@@ -839,7 +832,7 @@ __global__ void __launch_bounds__(BLOCK, TRACE || SPHERE || BRICKS || K >= 25 ? 
         if (cl.next >= kp.n) return;  // whole warp exits together
         cl.end = min(cl.next + kp.chunk, kp.n);
     }
-    walk_rays<K, PREC, TRACE, SPHERE, BRICKS>(kp, &kp.tree, nullptr, 1, nullptr, stack, cl);
+    walk_rays<K, PREC, TRACE, SPHERE, BRICKS>(kp, &kp.tree, nullptr, 1, stack, cl);
 }
 
 // ---------------------------------------------------------------- batched render
@@ -849,32 +842,25 @@ __global__ void __launch_bounds__(BLOCK, TRACE || SPHERE || BRICKS || K >= 25 ? 
 // balance themselves); lanes refill from the warp's claim as in k_render.
 // Leaf precision and SH degree are read from the tree table per ray.
 constexpr int MAX_BATCH = 16;
-constexpr int BATCH_TOP_NODES = 73;  // levels 0..2 of a full octree
+constexpr int BATCH_TOP_NODES = 73;  // levels 0..2 of a full octree (the configuration's largest top_nodes)
 
 struct BatchParams {
     KParams base;  // render parameters, outputs, cursor (base.tree unused)
     TreeParams trees[MAX_BATCH];
     int64_t off[MAX_BATCH + 1];
     int32_t n_trees;
-    int32_t stack_off;  // entries (uint2) of staged nodes before the node stack
 };
 
 template <bool BRICKS>
-__global__ void __launch_bounds__(BLOCK, 3)  // 4 blocks per SM spill: 4.6 against 3.4 ms (6 trees, 2.5M rays)
+__global__ void __launch_bounds__(BLOCK, 3)  // 4 blocks per SM spill: 2.64 against 2.45 ms (6 trees, 2.5M rays)
     k_render_batch(BatchParams bp) {
-    extern __shared__ uint2 s_nodes[];
+    extern __shared__ uint32_t s_stack[];  // per-thread node stack, as deep as the deepest tree needs
     __shared__ TreeParams s_tp[MAX_BATCH];
     __shared__ long long s_off[MAX_BATCH + 1];
     if (threadIdx.x < bp.n_trees) s_tp[threadIdx.x] = bp.trees[threadIdx.x];
     if (threadIdx.x <= bp.n_trees) s_off[threadIdx.x] = bp.off[threadIdx.x];
-    for (int t = 0; t < bp.n_trees; ++t) {
-        const TreeParams& tp = bp.trees[t];
-        for (int j = threadIdx.x; j < tp.n_top * 8; j += BLOCK) s_nodes[tp.s_off + j] = tp.nodes[j];
-    }
     __syncthreads();
-    // per-thread node stack after the staged nodes
-    uint32_t* stack = reinterpret_cast<uint32_t*>(s_nodes + bp.stack_off) + threadIdx.x;
-    walk_rays<0, -1, false, false, BRICKS>(bp.base, s_tp, s_off, bp.n_trees, s_nodes, stack,
+    walk_rays<0, -1, false, false, BRICKS>(bp.base, s_tp, s_off, bp.n_trees, s_stack + threadIdx.x,
                                            Claim{0, 0, true});
 }
 
@@ -973,8 +959,6 @@ void fill_tree_params(const plo_tree* t, const plo_render_params* p, TreeParams*
     tp->flags = t->d_flags;
     tp->sh_stride = t->sh_stride;
     tp->depth = t->depth;
-    tp->n_top = bricks ? t->n_top_staged : t->n_top;
-    tp->s_off = 0;
     tp->K = t->K;
     tp->prec = t->precision;
     tp->max_steps = p->max_steps > 0 ? p->max_steps : 4 * (1 << t->depth) + 64;
@@ -1416,7 +1400,6 @@ struct plo_batch {
     int sm_count;
     int device;
     plo_batch_config cfg;
-    int32_t full_top[MAX_BATCH];  // stageable top nodes per tree (<= BATCH_TOP_NODES)
     bool bricks;                  // some tree uses the brick layout
     unsigned long long* d_cursor;
     cudaGraph_t graph;
@@ -1426,18 +1409,9 @@ struct plo_batch {
 namespace {
 
 void apply_config(plo_batch* b) {
-    int32_t off = 0;
-    for (int t = 0; t < b->n_trees; ++t) {
-        const int32_t n = b->cfg.top_nodes > 0 ? std::min(b->full_top[t], b->cfg.top_nodes) : 0;
-        b->bp.trees[t].n_top = n;
-        b->bp.trees[t].s_off = off;
-        off += n * 8;
-    }
     int rows = 1;
     for (int t = 0; t < b->n_trees; ++t) rows = std::max(rows, b->bp.trees[t].top_depth + 1);
-    b->bp.stack_off = off;
-    b->smem = (size_t)off * sizeof(uint2) + (size_t)rows * BLOCK * 4;
-    b->bp.base.claim = b->cfg.claim_rays;
+    b->smem = (size_t)rows * BLOCK * 4;
 }
 
 void (*batch_kernel(const plo_batch* b))(BatchParams) {
@@ -1456,6 +1430,12 @@ cudaError_t launch_batch(plo_batch* b, cudaStream_t s) {
     int64_t warps_needed = (b->n_rays + 31) / 32;
     int64_t grid = std::min<int64_t>((warps_needed + WARPS - 1) / WARPS, (int64_t)b->sm_count * bps);
     if (grid < 1) return cudaSuccess;
+    // the configured claim is an upper bound: a warp's claims are at most a
+    // sixteenth of its even share, so that the end of the queue is spread over
+    // all warps (6 trees, 2.5M rays, claims of 256, 128, 64, 32: 2.77, 2.59,
+    // 2.49, 2.45 ms; 3 trees, 300k rays: 1.09, 0.64, 0.53, 0.46 ms)
+    const int64_t share = b->n_rays / (grid * WARPS * 16) / 32 * 32;
+    b->bp.base.claim = std::max<int64_t>(32, std::min<int64_t>(b->cfg.claim_rays, share));
     e = cudaMemsetAsync(b->d_cursor, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     fn<<<(unsigned)grid, BLOCK, b->smem, s>>>(b->bp);
@@ -1514,7 +1494,6 @@ extern "C" plo_status plo_batch_create(const plo_tree* const* trees, int32_t n_t
     for (int t = 0; t < n_trees; ++t) {
         fill_tree_params(trees[t], params, &b->bp.trees[t]);
         b->bricks |= trees[t]->layout == PLO_LAYOUT_BRICKS;
-        b->full_top[t] = std::min<int32_t>(b->bp.trees[t].n_top, BATCH_TOP_NODES);
     }
     for (int t = 0; t <= n_trees; ++t) b->bp.off[t] = ray_offsets[t];
     b->bp.n_trees = n_trees;
@@ -1615,27 +1594,25 @@ extern "C" plo_status plo_batch_autotune(plo_batch* b, const float* d_rays, floa
     float best_t = 1e30f;
     const int claims[] = {32, 64, 128, 256, 1024};
     const int bpss[] = {0, 1, 2};
-    const int tops[] = {0, BATCH_TOP_NODES};
     cudaError_t err = cudaSuccess;
     for (int ci = 0; ci < 5 && err == cudaSuccess; ++ci)
-        for (int bi = 0; bi < 3 && err == cudaSuccess; ++bi)
-            for (int ti = 0; ti < 2 && err == cudaSuccess; ++ti) {
-                b->cfg = {claims[ci], bpss[bi], tops[ti]};
-                apply_config(b);
-                err = launch_batch(b, s);  // warm-up
-                if (err != cudaSuccess) break;
-                cudaEventRecord(e0, s);
-                for (int r = 0; r < reps && err == cudaSuccess; ++r) err = launch_batch(b, s);
-                cudaEventRecord(e1, s);
-                cudaEventSynchronize(e1);
-                float ms = 0.0f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                ms /= (float)reps;
-                if (ms < best_t) {
-                    best_t = ms;
-                    best = b->cfg;
-                }
+        for (int bi = 0; bi < 3 && err == cudaSuccess; ++bi) {
+            b->cfg = {claims[ci], bpss[bi], saved.top_nodes};
+            apply_config(b);
+            err = launch_batch(b, s);  // warm-up
+            if (err != cudaSuccess) break;
+            cudaEventRecord(e0, s);
+            for (int r = 0; r < reps && err == cudaSuccess; ++r) err = launch_batch(b, s);
+            cudaEventRecord(e1, s);
+            cudaEventSynchronize(e1);
+            float ms = 0.0f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            ms /= (float)reps;
+            if (ms < best_t) {
+                best_t = ms;
+                best = b->cfg;
             }
+        }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     b->cfg = err == cudaSuccess ? best : saved;
