@@ -276,36 +276,40 @@ extern "C" plo_status plo_pt_render(const plo_tree* lum, const plo_render_params
         return cuda_error(e, "path tracer workspace");
     }
     float* samples = d_samples ? d_samples : own_samples;
-    a.ray = ws;
-    a.thr = a.ray + 6 * chunk;
+    // a bounce's next-event rays do not depend on the next bounce's own rays:
+    // both are one query of 2n rays (nee_ray, then ray), whose results follow
+    // each other the same way; a wavefront twice as large keeps the GPU busier
+    // (256 x 256 x 4 samples, 3 bounces, depth-8 luminaire: 1835 -> 1445 us)
+    a.thr = ws + 12 * chunk;
     a.L = a.thr + 3 * chunk;
-    a.nee_ray = a.L + 3 * chunk;
-    a.nee_w = a.nee_ray + 6 * chunk;
-    float* rgbA = a.nee_w + 3 * chunk;
-    float* TA = rgbA + 3 * chunk;
-    float* rgbB = TA + chunk;
-    float* TB = rgbB + 3 * chunk;
-    a.rgbA = rgbA;
-    a.TA = TA;
-    a.rgbB = rgbB;
+    a.nee_w = a.L + 3 * chunk;
+    float* rgb = a.nee_w + 3 * chunk;
+    float* T = rgb + 6 * chunk;
+    const bool octree = scene->emitter == PLO_PT_OCTREE;
     for (int64_t base = 0; st == PLO_OK && base < total; base += chunk) {
         a.base = base;
         a.n = total - base < chunk ? total - base : chunk;
+        a.nee_ray = ws;
+        a.ray = ws + 6 * a.n;
+        a.rgbB = rgb;
+        a.rgbA = rgb + 3 * a.n;
+        a.TA = T + a.n;
         const unsigned blocks = (unsigned)((a.n + 255) / 256);
+        auto query = [&](int64_t first, int64_t n) {  // rays first .. first + n of the two wavefronts
+            if (octree) {
+                st = plo_render_rays(lum, ws + 6 * first, n, params, rgb + 3 * first, T + first, nullptr, stream);
+            } else {
+                PtArgs q = a;
+                q.n = n;
+                k_pt_box_query<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(q, ws + 6 * first, rgb + 3 * first, T + first);
+            }
+        };
         k_pt_camera<<<blocks, 256, 0, s>>>(a);
+        query(a.n, a.n);
         for (int b = 0; st == PLO_OK && b < scene->max_bounces; ++b) {
-            if (scene->emitter == PLO_PT_OCTREE)
-                st = plo_render_rays(lum, a.ray, a.n, params, rgbA, TA, nullptr, stream);
-            else
-                k_pt_box_query<<<blocks, 256, 0, s>>>(a, a.ray, rgbA, TA);
-            if (st != PLO_OK) break;
             k_pt_wall<<<blocks, 256, 0, s>>>(a, b);
-            if (scene->emitter == PLO_PT_OCTREE)
-                st = plo_render_rays(lum, a.nee_ray, a.n, params, rgbB, TB, nullptr, stream);
-            else
-                k_pt_box_query<<<blocks, 256, 0, s>>>(a, a.nee_ray, rgbB, TB);
-            if (st != PLO_OK) break;
-            k_pt_nee<<<blocks, 256, 0, s>>>(a);
+            query(0, b + 1 < scene->max_bounces ? 2 * a.n : a.n);
+            if (st == PLO_OK) k_pt_nee<<<blocks, 256, 0, s>>>(a);
         }
         if (st == PLO_OK) k_pt_store<<<blocks, 256, 0, s>>>(a, samples);
     }

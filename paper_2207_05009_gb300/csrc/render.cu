@@ -1119,8 +1119,10 @@ __global__ void k_order_outputs(const uint32_t* inv, int64_t n, const float* rgb
 // Large wavefronts are handed out dynamically: warps claim RENDER_CLAIM rays
 // at a time from a counter allocated for the call, so a warp whose rays are
 // long does not hold up the end of the launch (static per-warp chunks are
-// kept below DYNAMIC_MIN_RAYS, where a call must not allocate).
-constexpr int64_t DYNAMIC_MIN_RAYS = (int64_t)1 << 20;
+// kept below DYNAMIC_MIN_RAYS, where they measure as fast and a call must not
+// allocate: 300,000, 400,000 and a million rays of the depth-8 luminaire take
+// 442, 545 and 1141 us with chunks, 457, 541 and 1082 us with the counter).
+constexpr int64_t DYNAMIC_MIN_RAYS = (int64_t)3 << 17;
 // Wavefronts of at least this many rays are also put in entry-cell order
 // (above): its fixed cost (a 5M-entry table per call) outweighs the gain on
 // smaller ones (measured on 2M rays of the depth-9 tree: 497 -> 468
