@@ -197,7 +197,8 @@ plo_status plo_tree_get_info(const plo_tree* tree, plo_tree_info* out);
  * gets PLO_RAY_STEP_LIMIT and raises the tree's device error flag (read by
  * plo_tree_check).  n == 0 is a no-op.  Calls with n >= 3 * 2^17 take an 8-byte
  * work counter from the stream-ordered allocator (cudaMallocAsync on
- * `stream`), so that warps claim rays dynamically. */
+ * `stream`), so that warps claim rays dynamically; below n = 2^20 a call whose
+ * stream is being captured, or that gets no memory, does without it. */
 plo_status plo_render_rays(const plo_tree* tree, const float* d_rays, int64_t n, const plo_render_params* params,
                            float* d_rgb, float* d_T, int32_t* d_status, void* stream);
 

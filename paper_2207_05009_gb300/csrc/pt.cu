@@ -263,9 +263,9 @@ extern "C" plo_status plo_pt_render(const plo_tree* lum, const plo_render_params
     a.dims = 2 + 5 * scene->max_bounces;
     const int64_t pixels = (int64_t)scene->width * scene->height;
     const int64_t total = pixels * spp;
-    const int64_t chunk = total < ((int64_t)1 << 22) ? total : ((int64_t)1 << 22);
+    const int64_t chunk = total < ((int64_t)1 << 21) ? total : ((int64_t)1 << 21);
     cudaStream_t s = (cudaStream_t)stream;
-    // workspace: ray, thr, L, nee_ray, nee_w, rgbA, TA, rgbB, TB (+ samples)
+    // workspace: nee_ray, ray, thr, L, nee_w, rgbB, rgbA, TB, TA (+ samples)
     const size_t per = 6 + 3 + 3 + 6 + 3 + 3 + 1 + 3 + 1;
     float* ws = nullptr;
     float* own_samples = nullptr;

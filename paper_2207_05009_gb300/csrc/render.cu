@@ -1123,6 +1123,10 @@ __global__ void k_order_outputs(const uint32_t* inv, int64_t n, const float* rgb
 // allocate: 300,000, 400,000 and a million rays of the depth-8 luminaire take
 // 442, 545 and 1141 us with chunks, 457, 541 and 1082 us with the counter).
 constexpr int64_t DYNAMIC_MIN_RAYS = (int64_t)3 << 17;
+// Below this many the chunks cost little, so a call that cannot have the
+// counter (no memory left) or should not (a captured graph with an allocation
+// in it can be instantiated only once) runs without it.
+constexpr int64_t DYNAMIC_ALWAYS_RAYS = (int64_t)1 << 20;
 // Wavefronts of at least this many rays are also put in entry-cell order
 // (above): its fixed cost (a 5M-entry table per call) outweighs the gain on
 // smaller ones (measured on 2M rays of the depth-9 tree: 497 -> 468
@@ -1170,15 +1174,26 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
     float *rgb_s = nullptr, *T_s = nullptr;
     int32_t* st_s = nullptr;
     const bool ordered = !TRACE && n >= ORDER_MIN_RAYS;
-    if (!TRACE && n >= DYNAMIC_MIN_RAYS && !ordered) {
+    bool counted = !TRACE && n >= DYNAMIC_MIN_RAYS && !ordered;
+    if (counted && n < DYNAMIC_ALWAYS_RAYS) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(cs, &capture) != cudaSuccess) cudaGetLastError();
+        counted = capture == cudaStreamCaptureStatusNone;
+    }
+    if (counted) {
         e = (cudaError_t)dev_malloc_async((void**)&cursor, sizeof(unsigned long long), cs);
-        if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), cs);
+        if (e == cudaErrorMemoryAllocation && n < DYNAMIC_ALWAYS_RAYS) {
+            cudaGetLastError();
+            cursor = nullptr;
+            e = cudaSuccess;
+        }
+        if (e == cudaSuccess && cursor) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), cs);
         if (e != cudaSuccess) {
             if (cursor) cudaFreeAsync(cursor, cs);
             return cuda_error(e, "render work counter");
         }
         kp.cursor = cursor;
-        kp.claim = RENDER_CLAIM;
+        kp.claim = cursor ? RENDER_CLAIM : kp.claim;
     }
     if (ordered) {
         // one scratch block: the claim counter, the (bin, block) table, the

@@ -65,3 +65,52 @@ def test_every_leaf_emits(cuda_available, n, act):
     rgb, T = _render(tree, rays, activation=act, l_max=3.0)
     ref = oracle.render(tree, rays, activation=oracle.SIGMOID if act == plo.ACT_SIGMOID else oracle.RELU, l_max=3.0)
     assert_radiance_close(rgb, T, ref, RTOL_FP32, what=f"{n} rays")
+
+
+def test_wavefront_sizes_and_the_work_counter(cuda_available):
+    """Each ray's arithmetic is its own, so a prefix of a wavefront gives the
+    same bits whatever the launch: one ray, fewer than a warp, spread out over
+    the SMs or not, with the work counter, without it because the allocation
+    failed, or captured in a graph."""
+    import torch
+    t = plo.Tree(plogen.luminaire_tree(plogen.LUMINAIRE_D6))
+    rays = torch.from_numpy(plogen.rays_sphere(3 << 17, seed=50)).cuda()
+    n = rays.shape[0]
+    rgb, T, _ = plo.render(t, rays)
+    torch.cuda.synchronize()
+    for m in (1, 31, 33, 2432, 2433, 77823, 77824, n - 1):
+        r, tr, _ = plo.render(t, rays[:m])
+        assert torch.equal(r, rgb[:m]) and torch.equal(tr, T[:m]), m
+    try:
+        plo.debug_fail_alloc_after(0)
+        r, tr, _ = plo.render(t, rays)
+    finally:
+        plo.debug_fail_alloc_after(-1)
+    assert torch.equal(r, rgb) and torch.equal(tr, T)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        r, tr, _ = plo.render(t, rays)
+    for _ in range(2):
+        r.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(r, rgb) and torch.equal(tr, T)
+    t.check()
+
+
+def test_batch_with_few_rays_per_warp(cuda_available):
+    """The claims of a batch shrink with its rays: a handful to 60,000 rays
+    over three trees equal the trees' own renders bit for bit."""
+    import torch
+    trees = [plo.Tree(plogen.luminaire_tree(plogen.LUMINAIRE_D6.with_(seed=s)), prec)
+             for s, prec in ((1, plo.PREC_FP32), (2, plo.PREC_FP16), (3, plo.PREC_BF16))]
+    for counts in ((1, 0, 2), (33, 5000, 1), (20000, 20001, 19999)):
+        offs = np.concatenate([[0], np.cumsum(counts)])
+        n = int(offs[-1])
+        rays = torch.from_numpy(plogen.rays_sphere(n, seed=60 + n)).cuda()
+        rgb, T = torch.full((n, 3), -1.0, device="cuda"), torch.full((n,), -1.0, device="cuda")
+        plo.Batch(trees, offs).render(rays, rgb, T)
+        for t, a, b in zip(trees, offs[:-1], offs[1:]):
+            if b > a:
+                r, tr, _ = plo.render(t, rays[a:b])
+                assert torch.equal(rgb[a:b], r) and torch.equal(T[a:b], tr), (counts, a)
