@@ -140,7 +140,7 @@ typedef struct {
 
 typedef struct {
     int32_t depth, sh_degree, precision;
-    int32_t top_levels;        /* levels staged in shared memory by the render kernel */
+    int32_t top_levels;        /* levels whose nodes come first in the node table       */
     int64_t n_nodes, n_leaves;
     int64_t n_sh_records;      /* leaves with at least one non-zero SH coefficient   */
     int64_t node_bytes;        /* device bytes of the node table                     */

@@ -301,7 +301,6 @@ plo_status pack_voxel_tree(int depth, int sh_degree, int precision, const uint32
     t->K = K;
     t->precision = precision;
     t->top_levels = T;
-    t->n_top = (int32_t)lv.n_top;
     t->n_nodes = n_nodes;
     t->n_leaves = nl;
     t->n_sh = nl;

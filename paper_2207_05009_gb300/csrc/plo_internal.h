@@ -51,7 +51,6 @@ constexpr uint32_t ENTRY_EMPTY = 0xFFFFFFFFu;
 constexpr uint32_t LEAF_BIT = 0x80000000u;
 constexpr uint32_t NO_SH_RECORD = 0x7FFFFFFEu;
 constexpr int MAX_DEPTH = 16;
-constexpr int MAX_TOP_NODES = 585;  // levels 0..3 of a full octree
 
 inline int sh_K(int degree) { return (degree + 1) * (degree + 1); }
 inline int sh_stride_bytes(int K, int precision) {
@@ -87,8 +86,7 @@ plo_status pack_voxel_tree(int depth, int sh_degree, int precision, const uint32
 struct plo_tree {
     int32_t depth;       // depth of the packed tree (>= 1; a root leaf is re-rooted one level down)
     int32_t sh_degree, K, precision;
-    int32_t top_levels;  // levels whose nodes are staged in shared memory
-    int32_t n_top;       // number of nodes in those levels (ids 0..n_top-1)
+    int32_t top_levels;  // levels whose nodes come first in the table, breadth-first
     int64_t n_nodes, n_leaves, n_sh;
     int32_t sh_stride;
     int32_t device;
@@ -104,7 +102,6 @@ struct plo_tree {
     int32_t layout;
     int32_t brick_log;     // brick side 2^brick_log finest cells
     int32_t brick_level;   // level of the brick cells (= depth for the octree layout)
-    int32_t n_top_staged;  // top-tree nodes of levels < min(4, brick_level)
     int64_t n_top_nodes, n_bricks;
     int64_t top_bytes, brick_bytes;
     void* d_top = nullptr;     // uint2 [n_top_nodes][8]

@@ -1000,9 +1000,9 @@ plo_status check_params(const plo_render_params* p) {
 // invalid are spread over the bins) moves the rays into a scratch copy, the render
 // kernel runs on the copy unchanged, and its outputs are moved back.
 // Neighbouring rays then walk neighbouring cells, so a warp's lanes share
-// node and record loads in L1 and L2 (measured on the 16M room rays of the
-// depth-10 tree, rays pre-sorted: 336.6 -> 356.6 Mrays/s with FP32 leaves,
-// 386.7 -> 400.8 with FP16; finer keys gained no more).  The sort keeps its
+// node and record loads in L1 and L2 (16M rays of the depth-10 tree with the
+// sort: 46.0 -> 40.8 ms with FP32 leaves, 39.6 -> 38.2 with FP16; finer keys
+// gained no more).  The sort keeps its
 // histograms in shared memory: one block per SM counts its contiguous chunk
 // of rays, a scan of the (bin, block) table gives every block its slot in
 // every bin, and the block scatters its chunk with shared-memory counters
@@ -1129,8 +1129,8 @@ constexpr int64_t DYNAMIC_MIN_RAYS = (int64_t)3 << 17;
 constexpr int64_t DYNAMIC_ALWAYS_RAYS = (int64_t)1 << 20;
 // Wavefronts of at least this many rays are also put in entry-cell order
 // (above): its fixed cost (a 5M-entry table per call) outweighs the gain on
-// smaller ones (measured on 2M rays of the depth-9 tree: 497 -> 468
-// Mrays/s with the order).
+// smaller ones (depth-9 luminaire, 3M rays: 4.63 -> 4.70 ms with the order;
+// 9M rays: the same with and without).
 constexpr int64_t ORDER_MIN_RAYS = (int64_t)1 << 23;
 
 template <bool TRACE>

@@ -220,7 +220,6 @@ plo_status build_tree(const plo_tree_desc* desc, const plo_build_options* opt, p
             new_id[nid] = (int32_t)order.size();
             order.push_back(nid);
         }
-    const int32_t n_top = (int32_t)order.size();
     // depth-first pre-order of the subtrees below the top levels
     std::vector<int32_t> stack;
     for (int32_t nid : bfs) {
@@ -353,14 +352,12 @@ plo_status build_tree(const plo_tree_desc* desc, const plo_build_options* opt, p
     std::vector<uint32_t> top_tab;
     std::vector<uint32_t> brick_cells;
     int64_t n_top_nodes = 0, n_bricks = 0;
-    int32_t n_top_staged = 0;
     if (bricks) {
         std::vector<int32_t> top_id(n_nodes, -1), brick_id(n_nodes, -1), top_order, brick_nodes;
         for (int32_t v : order) {
             if (level[v] < B) {
                 top_id[v] = (int32_t)top_order.size();
                 top_order.push_back(v);
-                if (level[v] < std::min(top, B)) ++n_top_staged;
             } else if (level[v] == B) {
                 brick_id[v] = (int32_t)brick_nodes.size();
                 brick_nodes.push_back(v);
@@ -429,7 +426,6 @@ plo_status build_tree(const plo_tree_desc* desc, const plo_build_options* opt, p
     t->brick_log = blog;
     t->brick_level = bricks ? B : depth;
     t->n_top_nodes = n_top_nodes;
-    t->n_top_staged = n_top_staged;
     t->n_bricks = n_bricks;
     t->top_bytes = n_top_nodes * 64;
     t->brick_bytes = (int64_t)brick_cells.size() * 4;
@@ -438,7 +434,6 @@ plo_status build_tree(const plo_tree_desc* desc, const plo_build_options* opt, p
     t->K = K;
     t->precision = precision;
     t->top_levels = top;
-    t->n_top = n_top;
     t->n_nodes = n_packed;
     t->n_leaves = desc->n_leaves;
     t->n_sh = n_sh;
