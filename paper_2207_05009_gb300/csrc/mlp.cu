@@ -2,10 +2,10 @@
 // library's own kernels on rays rendered from a ground-truth octree.
 //
 //   sampling + positional encoding  k_pe        (Sec. 4.1 ray marching, Sec. 4.2 PE)
-//   8 x 256 ReLU layers + SH head   k_gemm      (tcgen05, gemm.cuh)
+//   8 x 256 ReLU layers, SH head    k_trunk     (tcgen05, trunk.cuh; PLO_ARCH_PAPER's last two layers: k_gemm)
 //   quadrature, loss, d loss/d raw  k_quad      (Eq. 3-6, Eq. 7-9)
 //   weight and bias gradients       k_wgrad (bias: an extra MMA against ones)
-//   data gradients through ReLU     k_gemm (mask epilogue; the forward keeps the masks as bits)
+//   data gradients through ReLU     k_trunk (the forward keeps the masks as bits)
 //   Adam + exponential lr decay     k_adam      (Sec. 4.4)
 //
 // Activations are bf16 [samples][features] row-major; weights are kept as
@@ -103,6 +103,22 @@ plo_status make_store_map(CUtensorMap* m, const void* base, uint64_t rows, uint6
     cuuint32_t es[2] = {1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return set_error(PLO_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string(r) + ")");
+    return PLO_OK;
+}
+
+// fp32 raw outputs [rows][64] written by TMA stores in boxes of 32 columns x
+// 128 rows with the 128-byte swizzle.
+plo_status make_raw_map(CUtensorMap* m, const void* base, uint64_t rows) {
+    EncodeFn fn = encoder();
+    if (!fn) return set_error(PLO_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    cuuint64_t dims[2] = {OUT_PAD, rows};
+    cuuint64_t strides[1] = {OUT_PAD * 4};
+    cuuint32_t box[2] = {32, 128};
+    cuuint32_t es[2] = {1, 1};
+    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, es,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return set_error(PLO_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string(r) + ")");
     return PLO_OK;
@@ -882,6 +898,7 @@ struct plo_mlp {
     float* tsamp = nullptr;             // [cap] sample parameters (coarse pass)
     float* wts = nullptr;               // [cap] quadrature weights (coarse pass)
     float* ray_loss = nullptr;
+    CUtensorMap mapO_raw;  // the fp32 raw outputs (TMA stores)
     CUtensorMap mapA_H[MAX_LAYERS], mapA_dO, mapA_dZ[DEPTH], mapA_dZc;  // A operand boxes (128 rows)
     CUtensorMap mapW_H[MAX_LAYERS], mapW_dO, mapW_dZ[DEPTH], mapW_dZc;  // wgrad boxes (64 rows)
     CUtensorMap mapO_H[MAX_LAYERS], mapO_dZc;           // TMA-store boxes (32 x 32)
@@ -950,6 +967,7 @@ plo_status ensure_workspace(plo_mlp* m, int64_t samples, int rays) {
     if (st == PLO_OK && paper) st = make_store_map(&m->mapO_dZc, m->dZc, samples, COMB_PAD);
     for (int l = 1; l < m->n_layers && st == PLO_OK; ++l)
         st = make_store_map(&m->mapO_H[l], m->H[l], samples, m->geom.in_pad[l]);
+    if (st == PLO_OK) st = make_raw_map(&m->mapO_raw, m->raw, samples);
     if (st == PLO_OK) st = make_map(&m->mapA_dO, m->dO, samples, OUT_PAD, 128);
     if (st == PLO_OK) st = make_map(&m->mapW_dO, m->dO, samples, OUT_PAD, 64);
     for (int k = 0; k < DEPTH && st == PLO_OK; ++k) {
@@ -1060,24 +1078,25 @@ void padded_to_canonical(const plo_mlp* m, const std::vector<float>& p, float* c
 // writes fp32 raw outputs.  For training (`masks`), each ReLU layer also
 // writes which of its outputs are positive as bits (HB), the backward pass's
 // ReLU masks at 1/16 of the bytes of the activations.
-// The trunk (layers 0..7) runs as one layer-fused kernel (k_trunk): each
-// 128-row tile stays in shared memory from the encoding to H[8]; the layers'
+// The trunk (layers 0..7) and the linear head run as one layer-fused kernel
+// (k_trunk): a tile stays in shared memory from the encoding on; the layers'
 // outputs H[1..8] are stored for the backward pass and the activation hook
-// (`keep` false: only H[8], which the head reads).
-template <bool BWD, bool BITS, int XKB>
+// (`keep` false: none, or H[8], which PLO_ARCH_PAPER's last layers read).
+template <bool BWD, bool BITS, int XKB, bool HEAD>
 cudaError_t launch_trunk_kernel(const gemm::TrunkMaps& maps, const gemm::TrunkArgs& a, int sms, cudaStream_t s) {
     const size_t smem = gemm::trunk_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(gemm::k_trunk<BWD, BITS, XKB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(gemm::k_trunk<BWD, BITS, XKB, HEAD>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int tiles = (a.M + 2 * gemm::BM - 1) / (2 * gemm::BM);
     const int pairs = std::min(tiles, std::max(sms / 2, 1));
     if (pairs < 1) return cudaSuccess;
-    gemm::k_trunk<BWD, BITS, XKB><<<2 * pairs, gemm::TR_THREADS, smem, s>>>(maps, a);
+    gemm::k_trunk<BWD, BITS, XKB, HEAD><<<2 * pairs, gemm::TR_THREADS, smem, s>>>(maps, a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_trunk(plo_mlp* m, int64_t samples, bool masks, bool keep, cudaStream_t s) {
-    static_assert(gemm::TR_LAYERS == DEPTH && gemm::TR_N == WIDTH, "trunk shape");
+cudaError_t launch_trunk(plo_mlp* m, int64_t samples, bool masks, bool keep, float* out, cudaStream_t s) {
+    static_assert(gemm::TR_LAYERS == DEPTH && gemm::TR_N == WIDTH && gemm::TR_HEAD == OUT_PAD, "trunk shape");
     gemm::TrunkMaps maps;
     maps.x = m->mapA_H[0];
     gemm::TrunkArgs a{};
@@ -1087,11 +1106,19 @@ cudaError_t launch_trunk(plo_mlp* m, int64_t samples, bool masks, bool keep, cud
         a.bias[l] = bias_ptr(m, m->master, l);
         a.bits[l] = masks ? m->HB[l + 1] : nullptr;
     }
-    a.store = keep ? 0xFFu : 0x80u;
+    a.store = keep ? 0xFFu : m->arch == PLO_ARCH_PAPER ? 0x80u : 0u;
     a.err = m->d_err;
     a.M = (int)samples;
-    return masks ? launch_trunk_kernel<false, true, 1>(maps, a, m->sms, s)
-                 : launch_trunk_kernel<false, false, 1>(maps, a, m->sms, s);
+    if (m->arch == PLO_ARCH_PAPER)
+        return masks ? launch_trunk_kernel<false, true, 1, false>(maps, a, m->sms, s)
+                     : launch_trunk_kernel<false, false, 1, false>(maps, a, m->sms, s);
+    maps.raw = m->mapO_raw;
+    a.w[DEPTH] = m->W[DEPTH];
+    a.bias[DEPTH] = bias_ptr(m, m->master, DEPTH);
+    a.out = out;
+    a.n_out = m->n_out;
+    return masks ? launch_trunk_kernel<false, true, 1, true>(maps, a, m->sms, s)
+                 : launch_trunk_kernel<false, false, 1, true>(maps, a, m->sms, s);
 }
 
 // The data-gradient chain down to dZ[0], from the gradient at the layer after
@@ -1111,22 +1138,16 @@ cudaError_t launch_trunk_bwd(plo_mlp* m, int64_t samples, cudaStream_t s) {
     a.store = (1u << DEPTH) - 1u;
     a.err = m->d_err;
     a.M = (int)samples;
-    return paper ? launch_trunk_kernel<true, true, COMB_PAD / 64>(maps, a, m->sms, s)
-                 : launch_trunk_kernel<true, true, OUT_PAD / 64>(maps, a, m->sms, s);
+    return paper ? launch_trunk_kernel<true, true, COMB_PAD / 64, false>(maps, a, m->sms, s)
+                 : launch_trunk_kernel<true, true, OUT_PAD / 64, false>(maps, a, m->sms, s);
 }
 
-plo_status forward_layers(plo_mlp* m, int64_t samples, cudaStream_t s, bool masks = false, bool keep = true) {
-    gemm::EpiArgs ep{};
-    ep.err = m->d_err;
-    cudaError_t e = launch_trunk(m, samples, masks, keep, s);
-    ep.bits_out = nullptr;  // no ReLU after the head
-    if (e == cudaSuccess && m->arch == PLO_ARCH_LINEAR_HEAD) {
-        ep.bias = bias_ptr(m, m->master, DEPTH);
-        ep.out_f32 = m->raw;
-        ep.ldo = OUT_PAD;
-        e = launch_gemm<OUT_PAD, WIDTH>(m->mapA_H[DEPTH], m->mapW[DEPTH], nullptr, ep, gemm::EPI_BIAS_F32, (int)samples, m->sms,
-                                        s);
-    } else if (e == cudaSuccess) {
+plo_status forward_layers(plo_mlp* m, int64_t samples, cudaStream_t s, bool masks = false, bool keep = true,
+                          float* out = nullptr) {
+    cudaError_t e = launch_trunk(m, samples, masks, keep, out, s);
+    if (e == cudaSuccess && m->arch == PLO_ARCH_PAPER) {
+        gemm::EpiArgs ep{};
+        ep.err = m->d_err;
         // [ReLU features -> H[9] (bf16) | sigma block -> sraw (fp32)], then the
         // SH layer, whose zero row 0 picks up sigma from sraw
         ep.bias = bias_ptr(m, m->master, DEPTH);
@@ -1417,8 +1438,11 @@ extern "C" plo_status plo_mlp_forward(plo_mlp* m, const float* d_points, int64_t
     plo_status st = ensure_workspace(m, n, m->cap_rays);
     if (st != PLO_OK) return st;
     k_pe_points<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d_points, n, m->H[0]);
-    st = forward_layers(m, n, s);
-    if (st != PLO_OK) return st;
+    // the linear head's rows leave the trunk kernel without padding where the
+    // caller's buffer takes its 16-byte copies
+    const bool direct = m->arch == PLO_ARCH_LINEAR_HEAD && ((uintptr_t)d_raw & 15) == 0;
+    st = forward_layers(m, n, s, false, true, direct ? d_raw : nullptr);
+    if (st != PLO_OK || direct) return st;
     k_unpad_raw<<<(unsigned)((n * m->n_out + 1023) / 1024), 256, 0, s>>>(m->raw, n, m->n_out, d_raw);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PLO_OK : cuda_error(e, "raw output copy");

@@ -49,12 +49,13 @@ namespace gemm {
 
 constexpr int TR_LAYERS = 8;
 constexpr int TR_N = 256;
+constexpr int TR_HEAD = 64;  // outputs of the linear head (padded)
 constexpr int TR_WSTAGES = 5;
 constexpr int TR_WROWS = TR_N / 2;             // weight rows in each CTA of the pair
 constexpr int TR_WBYTES = TR_WROWS * 128;      // one K-block of half a weight matrix: 128 rows x 128 B
 constexpr int TR_KBYTES = BM * 128;            // one K-block of an activation tile: 128 rows x 128 B
 constexpr int TR_ABYTES = 4 * TR_KBYTES;       // a 128 x 256 bf16 activation tile
-constexpr int TR_BIAS_BYTES = TR_LAYERS * TR_N * 4;
+constexpr int TR_BIAS_BYTES = (TR_LAYERS * TR_N + TR_HEAD) * 4;
 constexpr int TR_BITS_BYTES = BM * TR_N / 8;   // ReLU bits of an activation tile: 128 rows x 32 B
 constexpr int TR_EPI_WARP0 = 4;
 constexpr int TR_EPI_GROUPS = 4;                      // epilogue warps per TMEM lane quadrant
@@ -72,11 +73,15 @@ struct TrunkMaps {
     CUtensorMap x;                 // input tile, boxes 64 x 128, 128-byte swizzle: the encoded samples [M][64]
                                    // (forward), the gradient after the trunk [M][64 XKB] (backward)
     CUtensorMap h[TR_LAYERS];      // job j's output [M][256], boxes 64 x 128 (TMA stores)
+    CUtensorMap raw;               // HEAD: the head's FP32 output [M][64], boxes 32 x 128, 128-byte swizzle
 };
 
 struct TrunkArgs {
-    const __nv_bfloat16* w[TR_LAYERS];  // B operand [256][K]: W_j (forward), W_l^T (backward); K = 64 XKB for j = 0
-    const float* bias[TR_LAYERS];  // forward: layer j's bias
+    const __nv_bfloat16* w[TR_LAYERS + 1];  // B operand [256][K]: W_j (forward; the head's last, [64][256]), W_l^T
+                                            // (backward); K = 64 XKB for j = 0
+    const float* bias[TR_LAYERS + 1];  // forward: layer j's bias
+    float* out;                    // HEAD: if not NULL the head's output goes here, [M][n_out], 16-byte aligned,
+    int n_out;                     // instead of through `raw`
     uint32_t* bits[TR_LAYERS];     // [M][8] words: forward, layer j's ReLU bits (written if BITS);
                                    // backward, the ReLU bits of H_l (read: the mask of the gradient)
     uint32_t store;                // bit j: store job j's output through h[j]
@@ -168,12 +173,14 @@ __device__ __forceinline__ uint32_t half_mask(uint32_t w) {
 // (dZ_l W_l) masked by the ReLU bits of H_l.  (A GEMM of its own for job 0
 // took 90 us per 524,288 rows, and the chain read its 268 MB back.)  BITS
 // (forward): write the layers' ReLU bits, which only a training step needs.
-// XKB: K-blocks of the input tile.
-template <bool BWD, bool BITS, int XKB>
+// XKB: K-blocks of the input tile.  HEAD (forward): the linear head (64
+// outputs, FP32, no ReLU) as a ninth job.
+template <bool BWD, bool BITS, int XKB, bool HEAD>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
     k_trunk(const __grid_constant__ TrunkMaps maps, TrunkArgs a) {
     constexpr uint32_t IDESC = sm100::idesc_bf16(2 * BM, TR_N, 0, 0);
-    constexpr int NJ = TR_LAYERS;  // jobs per tile
+    constexpr uint32_t IDESC_HEAD = sm100::idesc_bf16(2 * BM, TR_HEAD, 0, 0);
+    constexpr int NJ = TR_LAYERS + (HEAD ? 1 : 0);  // jobs per tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* act[2] = {smem, smem + TR_ABYTES};
@@ -207,7 +214,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
         sm100::fence_mbar_init();
     }
     if (!BWD)
-        for (int j = threadIdx.x; j < TR_LAYERS * TR_N; j += TR_THREADS) s_bias[j] = __ldg(a.bias[j / TR_N] + j % TR_N);
+        for (int j = threadIdx.x; j < TR_LAYERS * TR_N + (HEAD ? TR_HEAD : 0); j += TR_THREADS)
+            s_bias[j] = __ldg(a.bias[j / TR_N] + j % TR_N);
     if (warp == 1) sm100::tmem_alloc_pair(&ctl->tmem, 2 * TR_N);
     sm100::tc_fence_before();
     __syncthreads();
@@ -229,14 +237,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
         for (int r = 0; ok && r < rounds; ++r)
             for (int l = 0; ok && l < NJ; ++l) {
                 const int nkb = l == 0 ? XKB : 4;
+                const int rows = HEAD && l == TR_LAYERS ? TR_HEAD / 2 : TR_WROWS;
                 const uint8_t* src = reinterpret_cast<const uint8_t*>(a.w[l]) +
-                                     ((size_t)rank * TR_WROWS + r0) * (nkb * 128) + c * 16;
+                                     ((size_t)((int)rank * rows + r0)) * (nkb * 128) + c * 16;
                 for (int kb = 0; kb < nkb; ++kb, w.next()) {
                     ok = __all_sync(0xffffffffu, tr_wait(&ctl->wempty[w.s], w.ph ^ 1u, limit, ctl, a.err));
                     if (!ok) break;
                     const uint32_t dst = sm100::smem_addr(wbuf + (size_t)w.s * TR_WBYTES) + r0 * 128;
 #pragma unroll 8
-                    for (int i = 0; i < TR_WROWS / 4; ++i)  // row r0 + 4 i
+                    for (int i = 0; i < rows / 4; ++i)  // row r0 + 4 i
                         sm100::copy_async_16(dst + i * 512 + ((c ^ ((r0 + 4 * i) & 7)) << 4),
                                              src + (size_t)(4 * i) * (nkb * 128) + kb * 128);
                     sm100::copy_async_arrive(rank == 0 ? &ctl->kready[w.s] : &ctl->wfull[w.s]);
@@ -328,7 +337,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                         for (int k = 0; k < BK / 16; ++k) {
                             const uint64_t adesc = sm100::smem_desc_sw128(a0 + 32 * k, 16, 1024);
                             const uint64_t bdesc = sm100::smem_desc_sw128(b0 + 32 * k, 16, 1024);
-                            sm100::mma_bf16_pair(d, adesc, bdesc, IDESC, (kb | k) != 0);
+                            sm100::mma_bf16_pair(d, adesc, bdesc, HEAD && l == TR_LAYERS ? IDESC_HEAD : IDESC,
+                                                 (kb | k) != 0);
                         }
                         issued = true;
                         if (p == slots - 1) sm100::mma_commit_pair(&ctl->wempty[v.s]);
@@ -363,6 +373,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
             sm100::mbar_arrive_expect_tx(&ctl->mfull[p], bytes);
             sm100::bulk_load(s_bits + p * TR_BITS_BYTES, a.bits[l] + (size_t)row0 * (TR_N / 32), bytes, &ctl->mfull[p]);
         };
+        // the head's output: two boxes of the padded rows, or the packed
+        // rows as one copy (16 bytes at a time: of a last tile whose rows are
+        // not a multiple of four, the last 1 to 3 rows one value at a time)
+        auto store_head = [&](int p, int row0) {
+            if (!a.out) {
+                for (int c = 0; c < 2; ++c)
+                    sm100::tma_store_2d(&maps.raw, c * 32, row0, act[p] + (size_t)c * TR_KBYTES);
+            } else {
+                const int rows = min(BM, a.M - row0), whole = rows & ~3;
+                float* dst = a.out + (size_t)row0 * a.n_out;
+                const float* src = reinterpret_cast<const float*>(act[p]);
+                if (whole > 0) sm100::bulk_store(dst, src, (uint32_t)(whole * a.n_out * 4));
+                for (int i = whole * a.n_out; i < rows * a.n_out; ++i) dst[i] = src[i];
+            }
+            sm100::bulk_commit();
+            sm100::bulk_wait_read_0();
+        };
         load_mask(0, 0, 0);
         load_mask(0, 0, 1);
         for (int r = 0; ok && r < rounds; ++r)
@@ -376,6 +403,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                     }
                     load_mask(l + 1 < NJ ? r : r + 1, l + 1 < NJ ? l + 1 : 0, p);
                     const int row0 = (2 * tile + (int)rank) * BM;
+                    if (HEAD && l == TR_LAYERS) {
+                        if (row0 < a.M) store_head(p, row0);
+                        sm100::mbar_arrive(&ctl->sdone[p]);
+                        sm100::mbar_arrive(&ctl->xfree[p]);
+                        ++jobs[p];
+                        continue;
+                    }
                     constexpr bool bits = !BWD && BITS;
                     if ((((a.store >> l) & 1u) || bits) && row0 < a.M) {
                         if ((a.store >> l) & 1u)
@@ -413,6 +447,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                         (l > 0 && !tr_wait(&ctl->sdone[p], (uint32_t)(jobs[p] - 1) & 1u, limit, ctl, a.err))) {
                         ok = false;
                         break;
+                    }
+                    if (HEAD && l == TR_LAYERS) {
+                        sm100::tc_fence_after();
+                        constexpr int HC = TR_HEAD / TR_EPI_GROUPS;  // columns per epilogue warp
+                        static_assert(HC == 16, "tmem_ld16");
+                        float v[HC];
+                        sm100::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(p * TR_N + grp * HC), v);
+                        const float4* b4 = reinterpret_cast<const float4*>(s_bias + TR_LAYERS * TR_N + grp * HC);
+#pragma unroll
+                        for (int j = 0; j < HC / 4; ++j) {
+                            const float4 b = b4[j];
+                            v[4 * j] += b.x;
+                            v[4 * j + 1] += b.y;
+                            v[4 * j + 2] += b.z;
+                            v[4 * j + 3] += b.w;
+                        }
+                        if (a.out) {
+                            float* row = reinterpret_cast<float*>(act[p]) + rl * a.n_out + grp * HC;
+#pragma unroll
+                            for (int j = 0; j < HC; ++j)
+                                if (grp * HC + j < a.n_out) row[j] = v[j];
+                        } else {
+                            uint8_t* row = act[p] + (size_t)(grp >> 1) * TR_KBYTES + (size_t)rl * 128;
+#pragma unroll
+                            for (int u = 0; u < HC / 4; ++u)
+                                *reinterpret_cast<float4*>(row + ((((grp & 1) * 4 + u) ^ (rl & 7)) << 4)) =
+                                    make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+                        }
+                        sm100::fence_proxy_async();
+                        sm100::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) {
+                            sm100::mbar_arrive(&ctl->adone[p]);
+                            sm100::mbar_arrive_cluster(ready[p]);
+                        }
+                        ++jobs[p];
+                        continue;
                     }
                     uint2* bits = reinterpret_cast<uint2*>(s_bits + p * TR_BITS_BYTES + rl * (TR_N / 8)) + grp;
                     const uint2 mask = BWD ? *bits : make_uint2(0u, 0u);
