@@ -149,9 +149,8 @@ cudaError_t launch_gemm(const CUtensorMap& A, const CUtensorMap& B, const CUtens
 }
 
 // Weight gradients of the `n` layers of `jobs` (all with NIN inputs) over M
-// samples.  The samples are split so that the CTAs fill the SMs one to three
-// times over, more often only where a CTA still gets several thousand of
-// them: each adds its 128 x NIN sums with atomics.
+// samples, which are split over the CTAs: each adds its 128 x NIN sums with
+// atomics.
 template <int NIN>
 cudaError_t launch_wgrad(const gemm::WgradJobs& jobs, int n, int M, int sms, unsigned int* err, cudaStream_t s) {
     const size_t smem = gemm::wgrad_smem_bytes<NIN>();
@@ -163,7 +162,12 @@ cudaError_t launch_wgrad(const gemm::WgradJobs& jobs, int n, int M, int sms, uns
         out_tiles = std::max(out_tiles, t);
         tiles += t;
     }
-    const int waves = std::min(3, std::max(1, M / 65536));
+    // CTAs per SM: what fits at once (two with 64 inputs, whose pipeline takes
+    // half the shared memory).  Further waves repeat the set-up and the atomics:
+    // 524,288 rows of 256 x 256 86, 98, 110 us and 256 x 64 63, 57, 63 us
+    // with 1, 2, 3; the training step's seven layers with the head 1739, 1741, 1756
+    // us per step.
+    const int waves = std::min(NIN == 64 ? 2 : 1, std::max(1, M / 65536));
     const int blocks64 = M / 64;
     int n_chunks = std::max(1, std::min(waves * sms / tiles, blocks64));
     const int chunk = ((blocks64 + n_chunks - 1) / n_chunks) * 64;
