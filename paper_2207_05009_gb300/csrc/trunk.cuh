@@ -1,8 +1,9 @@
 // Layer-fused forward of the network's trunk (Sec. 4.2: eight fully
-// connected layers of 256 with ReLU) on sm_103a: a tile's activations stay in
-// shared memory from the encoded input to the eighth layer's output; only
-// what the backward pass needs leaves the SM (each layer's bf16 output,
-// stored by TMA straight from the shared-memory tile, and its ReLU bits).
+// connected layers of 256 with ReLU) and of the linear head on sm_103a: a
+// tile's activations stay in shared memory from the encoded input to the
+// head's output; only that and what the backward pass needs leaves the SM (each
+// layer's bf16 output, stored by TMA straight from the shared-memory tile, and
+// its ReLU bits).
 //
 // A pair of CTAs (a cluster of 2, tcgen05 cta_group::2) works on a tile of 256
 // rows, 128 in each, against the layer's 256 x K weights, half of whose rows
@@ -17,9 +18,10 @@
 // the biases and the ReLU bits: those used to be 4-byte accesses to global
 // memory in every epilogue.
 //
-// Measured on 524,288 rows (ncu): the forward 645 us with one CTA per tile,
-// now 515 us with ReLU bits and all layers stored and 375 us with neither;
-// seven data-gradient layers 495 us, now eight in 445 us.  The stores of 2.15
+// Measured on 524,288 rows (ncu): the forward 645 us with one CTA per tile and
+// the head 45 us as a GEMM that read its input back; the trunk alone now takes
+// 515 us with ReLU bits and all layers stored, with the head as a ninth job 556
+// us.  Seven data-gradient layers 495 us, now eight in 445 us.  The stores of 2.15
 // GB alone take 345 us at the rate the memory takes them, the MMAs alone 246
 // us (everything but them taken out), everything but the stores 400 us.  So
 // it is bound by its epilogue, whose warps serve the two slots in turn, and by
@@ -80,7 +82,7 @@ struct TrunkArgs {
     const __nv_bfloat16* w[TR_LAYERS + 1];  // B operand [256][K]: W_j (forward; the head's last, [64][256]), W_l^T
                                             // (backward); K = 64 XKB for j = 0
     const float* bias[TR_LAYERS + 1];  // forward: layer j's bias
-    float* out;                    // HEAD: if not NULL the head's output goes here, [M][n_out], 16-byte aligned,
+    float* out;                    // HEAD without BITS: if not NULL the head's output goes here, [M][n_out], 16-byte aligned,
     int n_out;                     // instead of through `raw`
     uint32_t* bits[TR_LAYERS];     // [M][8] words: forward, layer j's ReLU bits (written if BITS);
                                    // backward, the ReLU bits of H_l (read: the mask of the gradient)
@@ -377,7 +379,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
         // rows as one copy (16 bytes at a time: of a last tile whose rows are
         // not a multiple of four, the last 1 to 3 rows one value at a time)
         auto store_head = [&](int p, int row0) {
-            if (!a.out) {
+            if (BITS || !a.out) {
                 for (int c = 0; c < 2; ++c)
                     sm100::tma_store_2d(&maps.raw, c * 32, row0, act[p] + (size_t)c * TR_KBYTES);
             } else {
@@ -463,7 +465,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                             v[4 * j + 2] += b.z;
                             v[4 * j + 3] += b.w;
                         }
-                        if (a.out) {
+                        if (!BITS && a.out) {
                             float* row = reinterpret_cast<float*>(act[p]) + rl * a.n_out + grp * HC;
 #pragma unroll
                             for (int j = 0; j < HC; ++j)
