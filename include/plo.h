@@ -179,7 +179,9 @@ plo_status plo_build_tree(const plo_tree_desc* desc, int32_t precision, plo_tree
  * (for lookup and trace), so it takes node_bytes + brick_bytes. */
 plo_status plo_build_tree_ex(const plo_tree_desc* desc, const plo_build_options* options, plo_tree** out);
 
-/* Frees a tree (NULL is a no-op).  Synchronises the device first. */
+/* Frees a tree (NULL is a no-op) and the scratch memory that its calls kept (a
+ * pool of the tree's own, at most 128 MB while no call runs).  Synchronises the
+ * device first. */
 void plo_tree_free(plo_tree* tree);
 
 plo_status plo_tree_get_info(const plo_tree* tree, plo_tree_info* out);
@@ -196,8 +198,8 @@ plo_status plo_tree_get_info(const plo_tree* tree, plo_tree_info* out);
  * PLO_RAY_INVALID.  A ray that exceeds max_steps keeps its partial result,
  * gets PLO_RAY_STEP_LIMIT and raises the tree's device error flag (read by
  * plo_tree_check).  n == 0 is a no-op.  Calls with n >= 3 * 2^17 take an 8-byte
- * work counter from the stream-ordered allocator (cudaMallocAsync on
- * `stream`), so that warps claim rays dynamically; below n = 2^20 a call whose
+ * work counter from the tree's stream-ordered memory pool (on `stream`), so
+ * that warps claim rays dynamically; below n = 2^20 a call whose
  * stream is being captured, or that gets no memory, does without it. */
 plo_status plo_render_rays(const plo_tree* tree, const float* d_rays, int64_t n, const plo_render_params* params,
                            float* d_rgb, float* d_T, int32_t* d_status, void* stream);
@@ -274,9 +276,8 @@ plo_status plo_batch_capture(plo_batch* batch, const float* d_rays, float* d_rgb
                              void* stream);
 plo_status plo_batch_replay(plo_batch* batch, void* stream);
 
-/* Times every launch shape of a small grid (claim 32..1024, blocks per SM,
- * shared-memory staging on/off) on these buffers, `reps` launches each, and
- * keeps the fastest; returns it and its time per launch.  Synchronous. */
+/* Times every launch shape of a small grid (claim 32..1024, blocks per SM) on
+ * these buffers, `reps` launches each, and keeps the fastest; returns it and its time per launch.  Synchronous. */
 plo_status plo_batch_autotune(plo_batch* batch, const float* d_rays, float* d_rgb, float* d_T, int32_t reps,
                               void* stream, plo_batch_config* best, float* best_ms);
 

@@ -49,6 +49,42 @@ int dev_malloc_async(void** p, size_t bytes, cudaStream_t s) {
     return (int)cudaMallocAsync(p, bytes, s);
 }
 
+int tree_malloc_async(const plo_tree* t, void** p, size_t bytes, cudaStream_t s) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) return dev_malloc_async(p, bytes, s);  // the graph's memory
+    if (hook_fails()) {
+        *p = nullptr;
+        return (int)cudaErrorMemoryAllocation;
+    }
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(t->pool_mu);
+        if (!t->pool) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = t->device;
+            unsigned long long keep = POOL_KEEP;
+            if (cudaMemPoolCreate(&t->pool, &props) != cudaSuccess) {
+                t->pool = nullptr;
+                cudaGetLastError();
+            } else if (cudaMemPoolSetAttribute(t->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+                cudaGetLastError();
+            }
+        }
+        pool = t->pool;
+    }
+    if (!pool) return (int)cudaMallocAsync(p, bytes, s);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may not fit, or be in the way
+        cudaGetLastError();
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    }
+    return (int)e;
+}
+
 plo_status cuda_error(int err, const char* what) {
     cudaError_t e = static_cast<cudaError_t>(err);
     return set_error(e == cudaErrorMemoryAllocation ? PLO_ERR_OOM : PLO_ERR_CUDA,
@@ -91,7 +127,8 @@ extern "C" plo_status plo_render_rays_host(const plo_tree* tree, const float* h_
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(ready, user);
     for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(s[k], ready, 0);
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = (cudaError_t)dev_malloc_async((void**)&buf[k], per, s[k]);
+    for (int k = 0; k < (n > chunk ? 2 : 1) && e == cudaSuccess; ++k)
+        e = (cudaError_t)tree_malloc_async(tree, (void**)&buf[k], per, s[k]);
     if (e != cudaSuccess) st = cuda_error(e, "plo_render_rays_host setup");
     for (int64_t off = 0, c = 0; st == PLO_OK && off < n; off += chunk, ++c) {
         const int64_t m = std::min(chunk, n - off);

@@ -177,16 +177,17 @@ unsigned blocks_of(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t);
 
 }  // namespace
 
-cudaError_t device_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, cudaStream_t s) {
+cudaError_t device_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, cudaStream_t s, const plo_tree* t) {
     if (n <= 0) return cudaSuccess;
     const int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     uint32_t* sums = nullptr;
-    cudaError_t e = (cudaError_t)dev_malloc_async((void**)&sums, (size_t)nb * 4, s);
+    cudaError_t e = (cudaError_t)(t ? tree_malloc_async(t, (void**)&sums, (size_t)nb * 4, s)
+                                    : dev_malloc_async((void**)&sums, (size_t)nb * 4, s));
     if (e != cudaSuccess) return e;
     k_scan_tile<<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, sums);
     e = cudaGetLastError();
     if (e == cudaSuccess && nb > 1) {
-        e = device_exclusive_scan(sums, sums, nb, s);
+        e = device_exclusive_scan(sums, sums, nb, s, t);
         if (e == cudaSuccess) {
             k_scan_add<<<blocks_of(n), 256, 0, s>>>(out, n, sums);
             e = cudaGetLastError();

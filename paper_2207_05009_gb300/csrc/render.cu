@@ -1181,7 +1181,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
         counted = capture == cudaStreamCaptureStatusNone;
     }
     if (counted) {
-        e = (cudaError_t)dev_malloc_async((void**)&cursor, sizeof(unsigned long long), cs);
+        e = (cudaError_t)tree_malloc_async(t, (void**)&cursor, sizeof(unsigned long long), cs);
         if (e == cudaErrorMemoryAllocation && n < DYNAMIC_ALWAYS_RAYS) {
             cudaGetLastError();
             cursor = nullptr;
@@ -1207,7 +1207,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
         const size_t o_rays = o_inv + up((size_t)n * 4), o_rgb = o_rays + up((size_t)n * 24);
         const size_t o_T = o_rgb + up((size_t)n * 12), o_st = o_T + up((size_t)n * 4);
         const size_t o_bins = o_st + (d_status ? up((size_t)n * 4) : 0), total = o_bins + up((size_t)n * 2);
-        e = (cudaError_t)dev_malloc_async((void**)&cursor, total, cs);
+        e = (cudaError_t)tree_malloc_async(t, (void**)&cursor, total, cs);
         if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, 256, cs);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_order_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                        (int)ORDER_SMEM);
@@ -1227,7 +1227,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
             const float3 iext = make_float3(t->inv_ext[0], t->inv_ext[1], t->inv_ext[2]);
             k_order_count<<<nblk, ORDER_THREADS, ORDER_SMEM, cs>>>(d_rays, n, chunk, bmin, iext, bins, table);
             e = cudaGetLastError();
-            if (e == cudaSuccess) e = device_exclusive_scan(table, table, (int64_t)ORDER_BINS * nblk, cs);
+            if (e == cudaSuccess) e = device_exclusive_scan(table, table, (int64_t)ORDER_BINS * nblk, cs, t);
             if (e == cudaSuccess) {
                 k_order_scatter<<<nblk, ORDER_THREADS, ORDER_SMEM, cs>>>(n, chunk, bins, table, order, inv);
                 k_order_rays<<<(unsigned)((n + 255) / 256), 256, 0, cs>>>(d_rays, n, order, rays_s);
@@ -1284,7 +1284,7 @@ extern "C" plo_status plo_trace_rays(const plo_tree* tree, const float* d_rays, 
     if (n < 0) return set_error(PLO_ERR_INVALID_ARG, "n must be >= 0");
     if (n == 0) return PLO_OK;
     float* rgbT = nullptr;
-    cudaError_t e = (cudaError_t)dev_malloc_async((void**)&rgbT, (size_t)n * 4 * sizeof(float), (cudaStream_t)stream);
+    cudaError_t e = (cudaError_t)tree_malloc_async(tree, (void**)&rgbT, (size_t)n * 4 * sizeof(float), (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_error(e, "trace scratch allocation");
     plo_status st = render_common<true>(tree, d_rays, n, params, rgbT, rgbT + 3 * n, nullptr, max_cells, d_leaf,
                                         d_t, d_count, stream);
