@@ -20,7 +20,7 @@
 // emission evaluated for 32 leaves at a time from a per-warp queue (walk_rays).
 // Before, with double-float positions, staged top nodes and the emission
 // evaluated where a ray meets it (9M rays at depth 9, FP32 leaves / 2M at
-// depth 8, BF16 leaves, T < 1e-4 stop): 18.4 / 2.95 ms; now 12.7 / 1.95 ms.
+// depth 8, BF16 leaves, T < 1e-4 stop): 18.4 / 2.95 ms; now 12.6 / 1.88 ms.
 //
 // Numerics (no FP64 on the device):
 //   * Each axis is mirrored so that the ray goes up it.  The parameter at
