@@ -66,12 +66,16 @@ int tree_malloc_async(const plo_tree* t, void** p, size_t bytes, cudaStream_t s)
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = t->device;
             unsigned long long keep = POOL_KEEP;
+            // not an operation of a capture that another thread may be making
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
             if (cudaMemPoolCreate(&t->pool, &props) != cudaSuccess) {
                 t->pool = nullptr;
                 cudaGetLastError();
             } else if (cudaMemPoolSetAttribute(t->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
                 cudaGetLastError();
             }
+            cudaThreadExchangeStreamCaptureMode(&mode);
         }
         pool = t->pool;
     }

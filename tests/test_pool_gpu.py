@@ -63,3 +63,34 @@ def test_threads_and_streams_share_a_tree(cuda_available):
         t.join()
     assert not bad
     tree.check()
+
+
+def test_pool_is_made_while_another_thread_captures(cuda_available):
+    """The first call on a tree that needs scratch, from one thread, while
+    another is capturing a render of the same tree."""
+    import torch
+    tree = plo.Tree(plogen.luminaire_tree(plogen.LUMINAIRE_D6))
+    rays = torch.from_numpy(plogen.rays_sphere(500_000, seed=95)).cuda()
+    small = rays[:1000].clone()
+    plo.render(tree, small)
+    torch.cuda.synchronize()
+    rgb, T = torch.empty((1000, 3), device="cuda"), torch.empty(1000, device="cuda")
+    big, bigT = torch.empty((500_000, 3), device="cuda"), torch.empty(500_000, device="cuda")
+    stream = torch.cuda.Stream()
+
+    def first_call():
+        plo.render(tree, rays, rgb=big, T=bigT, stream=stream)
+        stream.synchronize()
+
+    graph = torch.cuda.CUDAGraph()
+    thread = threading.Thread(target=first_call)
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        plo.render(tree, small, rgb=rgb, T=T)
+        thread.start()
+        thread.join()
+    graph.replay()
+    torch.cuda.synchronize()
+    want, wantT, _ = plo.render(tree, rays)
+    torch.cuda.synchronize()
+    assert torch.equal(big, want) and torch.equal(bigT, wantT)
+    assert torch.equal(rgb, want[:1000]) and torch.equal(T, wantT[:1000])
