@@ -1743,7 +1743,9 @@ plo_status distill(plo_mlp* m, int32_t depth, int32_t samples, float sigma_thres
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t total = (int64_t)1 << (3 * depth);
     const int64_t C = total < ((int64_t)1 << 19) ? total : ((int64_t)1 << 19);
-    plo_status st = ensure_workspace(m, C < 128 ? 128 : C, m->cap_rays);
+    // pass 1 evaluates C voxels at a time, pass 2 the samples of at least one
+    // voxel, which are more than a shallow tree (depth 1 or 2) has voxels
+    plo_status st = ensure_workspace(m, std::max<int64_t>({C, samples, 128}), m->cap_rays);
     if (st != PLO_OK) return st;
     const int K = m->K;
     const int stride = sh_stride_bytes(K, precision);
