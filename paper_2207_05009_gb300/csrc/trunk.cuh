@@ -312,11 +312,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                 const int nkb = l == 0 ? XKB : 4;
                 TrStage v = w;
                 for (int p = 0; ok && p < slots; ++p) {
-                    // the input: the loaded tile, or the previous layer's output
-                    const bool in = l == 0 ? tr_wait(&ctl->xfull[p], (uint32_t)xs[p] & 1u, limit, ctl, a.err) &&
-                                                 tr_wait(&ctl->px[p], (uint32_t)xs[p] & 1u, limit, ctl, a.err)
-                                           : tr_wait(&ctl->aready[p], (uint32_t)(jobs[p] - 1) & 1u, limit, ctl, a.err);
-                    if (l == 0) ++xs[p];
+                    // the slot's previous job: its output is the input, or (l == 0) the epilogues are done
+                    // with its accumulator.  Every phase of aready is waited for, also that of a tile's last
+                    // job: a parity wait that skips one returns at once while the skipped one is incomplete.
+                    bool in = jobs[p] == 0 ||
+                              tr_wait(&ctl->aready[p], (uint32_t)(jobs[p] - 1) & 1u, limit, ctl, a.err);
+                    if (in && l == 0) {  // the loaded tile
+                        in = tr_wait(&ctl->xfull[p], (uint32_t)xs[p] & 1u, limit, ctl, a.err) &&
+                             tr_wait(&ctl->px[p], (uint32_t)xs[p] & 1u, limit, ctl, a.err);
+                        ++xs[p];
+                    }
                     if (!in) {
                         ok = false;
                         break;
