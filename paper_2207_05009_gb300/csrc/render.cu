@@ -615,7 +615,8 @@ __device__ __forceinline__ void leaf_step(const KParams& kp, const TreeParams& t
     const float seg = __fmaf_rn((float)(uint32_t)(dt >> 32), 3.7252902984619140625e-9f,  // 2^(32 - T_FRAC)
                                 (float)(uint32_t)dt * 8.673617379884035472e-19f) *       // 2^-T_FRAC
                       R.scale;
-    ++R.steps;
+    // the empty segment behind a hidden plane is no cell visited (the trace has none)
+    if (TRACE || seg > 0.0f) ++R.steps;
     if (TRACE) {
         auto param = [&](long long t) {  // caller's parameter, rounded once
             const float h = (float)(uint32_t)(t >> 37) * R.scale;  // 24 bits: exact
