@@ -202,7 +202,11 @@ __global__ void __launch_bounds__(32 * GRAD_WARPS) k_grad(GradArgs p) {
             Tn = lin ? fmaxf(0.0f, __fsub_rn(__fsub_rn(1.0f, hi), lo)) : expf(-(hi + lo));
             float T = __shfl_up_sync(ALL, Tn, 1);
             if (lane == 0) T = T_carry;
-            live = j < m && T > 0.0f;  // nothing behind T = 0 contributes
+            // nothing behind T = 0 contributes; a NaN (of an infinite optical depth) is no such end, and
+            // shows in the loss
+            const unsigned stop = __ballot_sync(ALL, j < m && Tn <= 0.0f);
+            const int at = stop ? __ffs(stop) - 1 : 31;
+            live = j < m && lane <= at;
             w = !live ? 0.0f : (lin ? fminf(T, a) : T * (-expm1f(-a)));
             emission();
             if (live) {
@@ -211,12 +215,10 @@ __global__ void __launch_bounds__(32 * GRAD_WARPS) k_grad(GradArgs p) {
                 alpha += w;
             }
             if (j < m) wt[j] = make_float2(w, live ? Tn : -1.0f);
-            const unsigned stop = __ballot_sync(ALL, live && Tn <= 0.0f);
             od_hi = __shfl_sync(ALL, hi, 31);
             od_lo = __shfl_sync(ALL, lo, 31);
             T_carry = __shfl_sync(ALL, Tn, 31);
             if (stop) {
-                const int at = __ffs(stop) - 1;
                 if (lin) {
                     sat = base + at;
 #pragma unroll
