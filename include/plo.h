@@ -179,9 +179,10 @@ plo_status plo_build_tree(const plo_tree_desc* desc, int32_t precision, plo_tree
  * (for lookup and trace), so it takes node_bytes + brick_bytes. */
 plo_status plo_build_tree_ex(const plo_tree_desc* desc, const plo_build_options* options, plo_tree** out);
 
-/* Frees a tree (NULL is a no-op) and the scratch memory that its calls kept (a
- * pool of the tree's own, at most 128 MB while no call runs).  Synchronises the
- * device first. */
+/* Frees a tree (NULL is a no-op).  Synchronises the device first.  The trees of
+ * a device share a pool of scratch memory, which goes with the last of them; it
+ * keeps at most 128 MB while no call runs, and gives those back when an
+ * allocation of this library finds no memory. */
 void plo_tree_free(plo_tree* tree);
 
 plo_status plo_tree_get_info(const plo_tree* tree, plo_tree_info* out);
@@ -198,7 +199,7 @@ plo_status plo_tree_get_info(const plo_tree* tree, plo_tree_info* out);
  * PLO_RAY_INVALID.  A ray that exceeds max_steps keeps its partial result,
  * gets PLO_RAY_STEP_LIMIT and raises the tree's device error flag (read by
  * plo_tree_check).  n == 0 is a no-op.  Calls with n >= 3 * 2^17 take an 8-byte
- * work counter from the tree's stream-ordered memory pool (on `stream`), so
+ * work counter from the trees' stream-ordered memory pool (on `stream`), so
  * that warps claim rays dynamically; below n = 2^20 a call whose
  * stream is being captured, or that gets no memory, does without it. */
 plo_status plo_render_rays(const plo_tree* tree, const float* d_rays, int64_t n, const plo_render_params* params,
@@ -565,7 +566,7 @@ typedef struct {
  *               or NULL to draw them from `seed` (SplitMix64)
  *   d_image     float [height][width][3]: mean radiance over the samples
  *   d_samples   float [spp][height][width][3] per-sample radiance, or NULL
- * Allocates its wavefront buffers with cudaMallocAsync on `stream`. */
+ * Allocates its wavefront buffers on `stream`, from the trees' scratch pool. */
 plo_status plo_pt_render(const plo_tree* lum, const plo_render_params* params, const plo_pt_scene* scene,
                          int32_t spp, uint64_t seed, const float* d_uniforms, float* d_image, float* d_samples,
                          void* stream);

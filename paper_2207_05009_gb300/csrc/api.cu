@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <mutex>
 #include <string>
 
 #include "plo_internal.h"
@@ -33,12 +34,91 @@ bool hook_fails() {
 }
 }  // namespace
 
+namespace {
+
+// The scratch pool of a device: made for the first tree there that needs it,
+// destroyed with the last one that used it.
+struct ScratchPool {
+    cudaMemPool_t pool = nullptr;
+    int64_t users = 0;  // trees
+};
+constexpr int MAX_DEVICES = 64;
+ScratchPool g_pools[MAX_DEVICES];
+std::mutex g_pools_mu;  // of g_pools and of every tree's `pool`
+
+// While one lives, this thread's calls on a pool are no operations of a
+// capture that another thread may be making.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// The pool for `t`'s scratch; null if none can be made.
+cudaMemPool_t scratch_pool(const plo_tree* t) {
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    if (t->pool) return t->pool;
+    if (t->device < 0 || t->device >= MAX_DEVICES) return nullptr;
+    ScratchPool& d = g_pools[t->device];
+    if (!d.pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = t->device;
+        unsigned long long keep = POOL_KEEP;
+        RelaxedCapture relaxed;
+        if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
+            d.pool = nullptr;
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+    }
+    ++d.users;
+    return t->pool = d.pool;
+}
+
+// Gives back what the device's pool keeps and does not need now.
+void trim_scratch(int device) {
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    if (device < 0 || device >= MAX_DEVICES || !g_pools[device].pool) return;
+    RelaxedCapture relaxed;
+    if (cudaMemPoolTrimTo(g_pools[device].pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
+// An allocation that found no memory is tried once more without what the
+// scratch pool keeps.
+template <class F>
+cudaError_t with_trim(F alloc) {
+    cudaError_t e = alloc();
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        int device = -1;
+        if (cudaGetDevice(&device) == cudaSuccess) trim_scratch(device);
+        e = alloc();
+    }
+    return e;
+}
+
+}  // namespace
+
+void release_scratch_pool(plo_tree* t) {
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    if (!t->pool) return;
+    ScratchPool& d = g_pools[t->device];
+    t->pool = nullptr;
+    if (--d.users == 0) {
+        cudaMemPoolDestroy(d.pool);
+        d.pool = nullptr;
+    }
+}
+
 int dev_malloc(void** p, size_t bytes) {
     if (hook_fails()) {
         *p = nullptr;
         return (int)cudaErrorMemoryAllocation;
     }
-    return (int)cudaMalloc(p, bytes);
+    return (int)with_trim([&] { return cudaMalloc(p, bytes); });
 }
 
 int dev_malloc_async(void** p, size_t bytes, cudaStream_t s) {
@@ -46,7 +126,7 @@ int dev_malloc_async(void** p, size_t bytes, cudaStream_t s) {
         *p = nullptr;
         return (int)cudaErrorMemoryAllocation;
     }
-    return (int)cudaMallocAsync(p, bytes, s);
+    return (int)with_trim([&] { return cudaMallocAsync(p, bytes, s); });
 }
 
 int tree_malloc_async(const plo_tree* t, void** p, size_t bytes, cudaStream_t s) {
@@ -57,36 +137,10 @@ int tree_malloc_async(const plo_tree* t, void** p, size_t bytes, cudaStream_t s)
         *p = nullptr;
         return (int)cudaErrorMemoryAllocation;
     }
-    cudaMemPool_t pool = nullptr;
-    {
-        std::lock_guard<std::mutex> lock(t->pool_mu);
-        if (!t->pool) {
-            cudaMemPoolProps props = {};
-            props.allocType = cudaMemAllocationTypePinned;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = t->device;
-            unsigned long long keep = POOL_KEEP;
-            // not an operation of a capture that another thread may be making
-            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            if (cudaMemPoolCreate(&t->pool, &props) != cudaSuccess) {
-                t->pool = nullptr;
-                cudaGetLastError();
-            } else if (cudaMemPoolSetAttribute(t->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-                cudaGetLastError();
-            }
-            cudaThreadExchangeStreamCaptureMode(&mode);
-        }
-        pool = t->pool;
-    }
-    if (!pool) return (int)cudaMallocAsync(p, bytes, s);
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may not fit, or be in the way
-        cudaGetLastError();
-        cudaMemPoolTrimTo(pool, 0);
-        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    }
-    return (int)e;
+    const cudaMemPool_t pool = scratch_pool(t);
+    return (int)with_trim([&] {  // what the pool keeps may not fit, or be in the way
+        return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+    });
 }
 
 plo_status cuda_error(int err, const char* what) {

@@ -41,7 +41,6 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <mutex>
 #include <string>
 
 #include "../../include/plo.h"
@@ -52,8 +51,9 @@ constexpr uint32_t ENTRY_EMPTY = 0xFFFFFFFFu;
 constexpr uint32_t LEAF_BIT = 0x80000000u;
 constexpr uint32_t NO_SH_RECORD = 0x7FFFFFFEu;
 constexpr int MAX_DEPTH = 16;
-// Scratch a tree's pool holds on to between calls: two chunks of 2^20 host rays
-// (84 MB), or the path tracer's workspace of a million samples.
+// Scratch that the trees of a device hold on to between calls, all together: two
+// chunks of 2^20 host rays (84 MB), or the path tracer's workspace of a million
+// samples.
 constexpr unsigned long long POOL_KEEP = 128ull << 20;
 
 inline int sh_K(int degree) { return (degree + 1) * (degree + 1); }
@@ -71,9 +71,12 @@ plo_status cuda_error(int err, const char* what);
 // n-th one fail (plo_debug_fail_alloc_after).
 int dev_malloc(void** p, size_t bytes);
 int dev_malloc_async(void** p, size_t bytes, cudaStream_t s);
-// The same from the tree's own pool (see plo_tree::pool), freed with
-// cudaFreeAsync: what a call on the tree needs while it runs.
+// The same from the scratch pool of the tree's device (see plo_tree::pool), freed
+// with cudaFreeAsync: what a call on the tree needs while it runs.  All three
+// give back what that pool keeps, and try once more, where no memory is left.
 int tree_malloc_async(const plo_tree* t, void** p, size_t bytes, cudaStream_t s);
+// The tree's use of the pool ends; the last use's end destroys it.
+void release_scratch_pool(plo_tree* t);
 
 // Exclusive prefix sum of n uint32 values on the device (async on s; its
 // temporary goes through tree_malloc_async with a tree, dev_malloc_async
@@ -119,8 +122,8 @@ struct plo_tree {
     // memory back at each synchronisation, so that a caller who waits for one
     // call before the next paid for mapping it again every time: renders of
     // 500,000 and 2,000,000 rays at depth 8 854 -> 669 and 2165 -> 1990 us, of
-    // 60,000 from host memory 468 -> 301 us.  This pool keeps POOL_KEEP bytes;
-    // it is made by the first call that needs it and goes with the tree.
+    // 60,000 from host memory 468 -> 301 us.  So the trees of a device share a
+    // pool that keeps POOL_KEEP bytes, however many trees there are; it is made
+    // for the first call that needs it and goes with the last tree that used it.
     mutable cudaMemPool_t pool = nullptr;
-    mutable std::mutex pool_mu;
 };

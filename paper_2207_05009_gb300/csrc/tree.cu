@@ -513,7 +513,7 @@ extern "C" void plo_tree_free(plo_tree* t) {
     cudaFree(t->d_flags);
     cudaFree(t->d_top);
     cudaFree(t->d_bricks);
-    if (t->pool) cudaMemPoolDestroy(t->pool);
+    release_scratch_pool(t);
     if (prev >= 0) cudaSetDevice(prev);
     delete t;
 }
