@@ -46,8 +46,9 @@ constexpr int MAX_DEVICES = 64;
 ScratchPool g_pools[MAX_DEVICES];
 std::mutex g_pools_mu;  // of g_pools and of every tree's `pool`
 
-// While one lives, this thread's calls on a pool are no operations of a
-// capture that another thread may be making.
+// While one lives, this thread's calls on pools and their memory are allowed
+// whatever another thread may be capturing (a capture in the global mode
+// forbids them to every thread, and ends in an error if one is made).
 struct RelaxedCapture {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
@@ -138,9 +139,16 @@ int tree_malloc_async(const plo_tree* t, void** p, size_t bytes, cudaStream_t s)
         return (int)cudaErrorMemoryAllocation;
     }
     const cudaMemPool_t pool = scratch_pool(t);
+    RelaxedCapture relaxed;
     return (int)with_trim([&] {  // what the pool keeps may not fit, or be in the way
         return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
     });
+}
+
+void scratch_free_async(void* p, cudaStream_t s) {
+    if (!p) return;
+    RelaxedCapture relaxed;
+    cudaFreeAsync(p, s);
 }
 
 plo_status cuda_error(int err, const char* what) {
@@ -204,7 +212,7 @@ extern "C" plo_status plo_render_rays_host(const plo_tree* tree, const float* h_
         if (e != cudaSuccess) { st = cuda_error(e, "device-to-host result copy"); break; }
     }
     for (int k = 0; k < 2; ++k) {
-        if (buf[k]) cudaFreeAsync(buf[k], s[k]);
+        scratch_free_async(buf[k], s[k]);
         if (s[k]) {
             cudaError_t se = cudaStreamSynchronize(s[k]);
             if (se != cudaSuccess && st == PLO_OK) st = cuda_error(se, "plo_render_rays_host");

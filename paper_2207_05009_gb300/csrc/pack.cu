@@ -193,7 +193,7 @@ cudaError_t device_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, 
             e = cudaGetLastError();
         }
     }
-    cudaFreeAsync(sums, s);
+    scratch_free_async(sums, s);
     return e;
 }
 

@@ -71,10 +71,13 @@ plo_status cuda_error(int err, const char* what);
 // n-th one fail (plo_debug_fail_alloc_after).
 int dev_malloc(void** p, size_t bytes);
 int dev_malloc_async(void** p, size_t bytes, cudaStream_t s);
-// The same from the scratch pool of the tree's device (see plo_tree::pool), freed
-// with cudaFreeAsync: what a call on the tree needs while it runs.  All three
-// give back what that pool keeps, and try once more, where no memory is left.
+// The same from the scratch pool of the tree's device (see plo_tree::pool): what
+// a call on the tree needs while it runs, also one beside another thread's
+// capture.  All three give back what that pool keeps, and try once more, where
+// no memory is left.
 int tree_malloc_async(const plo_tree* t, void** p, size_t bytes, cudaStream_t s);
+// Frees what either of the stream-ordered ones gave (NULL is a no-op).
+void scratch_free_async(void* p, cudaStream_t s);
 // The tree's use of the pool ends; the last use's end destroys it.
 void release_scratch_pool(plo_tree* t);
 

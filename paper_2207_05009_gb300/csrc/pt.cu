@@ -272,7 +272,7 @@ extern "C" plo_status plo_pt_render(const plo_tree* lum, const plo_render_params
     cudaError_t e = (cudaError_t)tree_malloc_async(lum, (void**)&ws, (size_t)chunk * per * 4, s);
     if (e == cudaSuccess && !d_samples) e = (cudaError_t)tree_malloc_async(lum, (void**)&own_samples, (size_t)total * 12, s);
     if (e != cudaSuccess) {
-        if (ws) cudaFreeAsync(ws, s);
+        scratch_free_async(ws, s);
         return cuda_error(e, "path tracer workspace");
     }
     float* samples = d_samples ? d_samples : own_samples;
@@ -315,8 +315,8 @@ extern "C" plo_status plo_pt_render(const plo_tree* lum, const plo_render_params
     }
     if (st == PLO_OK) k_pt_resolve<<<(unsigned)((pixels + 255) / 256), 256, 0, s>>>(samples, pixels, spp, d_image);
     e = cudaGetLastError();
-    cudaFreeAsync(ws, s);
-    if (own_samples) cudaFreeAsync(own_samples, s);
+    scratch_free_async(ws, s);
+    scratch_free_async(own_samples, s);
     if (st != PLO_OK) return st;
     return e == cudaSuccess ? PLO_OK : cuda_error(e, "path tracer launch");
 }

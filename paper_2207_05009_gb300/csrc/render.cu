@@ -1190,7 +1190,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
         }
         if (e == cudaSuccess && cursor) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), cs);
         if (e != cudaSuccess) {
-            if (cursor) cudaFreeAsync(cursor, cs);
+            scratch_free_async(cursor, cs);
             return cuda_error(e, "render work counter");
         }
         kp.cursor = cursor;
@@ -1240,7 +1240,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
             kp.status = st_s;
         }
         if (e != cudaSuccess) {
-            if (cursor) cudaFreeAsync(cursor, cs);
+            scratch_free_async(cursor, cs);
             return cuda_error(e, "render work counter and ray order");
         }
         kp.cursor = cursor;
@@ -1259,7 +1259,7 @@ plo_status render_common(const plo_tree* t, const float* d_rays, int64_t n, cons
         k_order_outputs<<<(unsigned)((n + 255) / 256), 256, 0, cs>>>(inv, n, rgb_s, T_s, st_s, d_rgb, d_T, d_status);
         e = cudaGetLastError();
     }
-    if (cursor) cudaFreeAsync(cursor, cs);
+    scratch_free_async(cursor, cs);
     if (e != cudaSuccess) return cuda_error(e, "render kernel launch");
     return PLO_OK;
 }
@@ -1289,7 +1289,7 @@ extern "C" plo_status plo_trace_rays(const plo_tree* tree, const float* d_rays, 
     if (e != cudaSuccess) return cuda_error(e, "trace scratch allocation");
     plo_status st = render_common<true>(tree, d_rays, n, params, rgbT, rgbT + 3 * n, nullptr, max_cells, d_leaf,
                                         d_t, d_count, stream);
-    cudaFreeAsync(rgbT, (cudaStream_t)stream);
+    scratch_free_async(rgbT, (cudaStream_t)stream);
     return st;
 }
 
