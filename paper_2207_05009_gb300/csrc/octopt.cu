@@ -445,19 +445,19 @@ __global__ void k_nb_from_lookup(const int64_t* leaf, int64_t n, int32_t* nb) {
 unsigned grid_of(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 template <int K>
-cudaError_t launch_grad(const GradArgs& a, cudaStream_t s) {
-    const unsigned blocks = std::min<unsigned>(grid_of(a.n, GRAD_WARPS), 12u * 152u);
+cudaError_t launch_grad(const GradArgs& a, int sms, cudaStream_t s) {
+    const unsigned blocks = std::min<unsigned>(grid_of(a.n, GRAD_WARPS), 12u * (unsigned)sms);
     k_grad<K><<<blocks, 32 * GRAD_WARPS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t dispatch_grad(int K, const GradArgs& a, cudaStream_t s) {
+cudaError_t dispatch_grad(int K, const GradArgs& a, int sms, cudaStream_t s) {
     switch (K) {
-        case 1: return launch_grad<1>(a, s);
-        case 4: return launch_grad<4>(a, s);
-        case 9: return launch_grad<9>(a, s);
-        case 16: return launch_grad<16>(a, s);
-        case 25: return launch_grad<25>(a, s);
+        case 1: return launch_grad<1>(a, sms, s);
+        case 4: return launch_grad<4>(a, sms, s);
+        case 9: return launch_grad<9>(a, sms, s);
+        case 16: return launch_grad<16>(a, sms, s);
+        case 25: return launch_grad<25>(a, sms, s);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -712,7 +712,7 @@ plo_status run_grad(plo_octopt* o, const float* d_rays, const float* d_rgb_gt, c
         }
         const int K = q == 0 ? 1 : o->K;
         const unsigned blocks = grid_of(nl * K, THREADS);
-        const unsigned terms_blocks = std::min<unsigned>(blocks, 8u * 152u);
+        const unsigned terms_blocks = std::min<unsigned>(blocks, 8u * (unsigned)o->walk->sm_count);
         const float scale = lam[q] / (float)nl;
         if (q == 0) {
             k_tv_terms<1><<<terms_blocks, THREADS, 0, o->side>>>(xs[q], K, o->d_nb, nl, o->d_tv_s, o->d_tv_own,
@@ -759,7 +759,7 @@ plo_status run_grad(plo_octopt* o, const float* d_rays, const float* d_rgb_gt, c
         a.l_max = o->cfg.l_max;
         a.eps = o->cfg.eps;
         a.inv_n = 1.0f / (float)n;
-        e = dispatch_grad(o->K, a, s);
+        e = dispatch_grad(o->K, a, o->walk->sm_count, s);
         if (e != cudaSuccess) return cuda_error(e, "gradient kernel launch");
     }
     if (d_loss_out) {
