@@ -253,7 +253,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TR_THREADS, 1)
                     sm100::copy_async_arrive(rank == 0 ? &ctl->kready[w.s] : &ctl->wfull[w.s]);
                 }
             }
-        sm100::copy_async_wait_all();  // nothing is in flight when the CTA exits
+        sm100::copy_async_wait_all();  // nothing is in flight when the CTA exits,
+#pragma unroll 1
+        for (int i = 0; ok && lane == 0 && i < TR_WSTAGES; ++i, w.next())  // nor the last MMAs' arrivals here
+            ok = tr_wait(&ctl->wempty[w.s], w.ph ^ 1u, limit, ctl, a.err);
     } else if (warp == 3 && lane == 0) {
         // ---------------- input tiles
         sm100::prefetch_tmap(&maps.x);
