@@ -166,7 +166,9 @@ cudaError_t launch_wgrad(const gemm::WgradJobs& jobs, int n, int M, int sms, uns
     // half the shared memory).  Further waves repeat the set-up and the atomics:
     // 524,288 rows of 256 x 256 86, 98, 110 us and 256 x 64 63, 57, 63 us
     // with 1, 2, 3; the training step's seven layers with the head 1739, 1741, 1756
-    // us per step.
+    // us per step.  With 64 inputs the second CTA pays from 131,072 rows on
+    // (256 x 64 of 16,384, 65,536, 98,304 and 131,072 rows, one against two: 8.8 /
+    // 11.4, 14.4 / 16.5, 18.8 / 20.6, 22.7 / 22.7 us).
     const int waves = std::min(NIN == 64 ? 2 : 1, std::max(1, M / 65536));
     const int blocks64 = M / 64;
     int n_chunks = std::max(1, std::min(waves * sms / tiles, blocks64));
@@ -1767,7 +1769,7 @@ plo_status distill(plo_mlp* m, int32_t depth, int32_t samples, float sigma_thres
     for (int64_t base = 0; e == cudaSuccess && st == PLO_OK && base < total; base += C) {
         const int64_t n = total - base < C ? total - base : C;
         k_pe_centres<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((uint64_t)base, n, depth, m->H[0]);
-        st = forward_layers(m, n, s, false, false);  // only H[8] is read (by the head)
+        st = forward_layers(m, n, s, false, false);  // no layer's output is stored that no kernel reads
         if (st != PLO_OK) break;
         k_keep<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(m->raw, n, sigma_thresh, d_flag);
         e = device_exclusive_scan(d_flag, d_pos, n, s);

@@ -12,8 +12,8 @@
 // coordinates on the finest grid.
 //
 // What bounds it: the latency of the dependent node loads, then instruction
-// issue (65% of the issue slots, depth-9 luminaire, 2M rays), at a tenth of
-// the DRAM bandwidth.  So the walk is built to need few instructions per cell
+// issue (64% of the issue slots, depth-9 luminaire, 2M rays), at 15% of the
+// DRAM bandwidth.  So the walk is built to need few instructions per cell
 // and little shared memory (what is left is L1): fixed-point plane parameters
 // (below), no staging of the top nodes (the test for it cost more than the
 // L1 hits it saved: 18.7 against 16.5 ms for 9M rays at depth 9), and SH
@@ -587,11 +587,12 @@ __device__ __forceinline__ float composite(const KParams& kp, Ray& R, float sigm
 //
 // The cell's three upper faces are finest-grid planes, so their parameters
 // are one 64-bit multiply-add each, and the segment is the difference of two
-// of them: exact to 2^-60, rounded once to FP32.  On the axes the ray does
+// of them, rounded once to FP32: exact to 2^-60 between planes of one axis, to
+// the set-up's double-float error (~2^-46) between two axes.  On the axes the ray does
 // not leave by, the next cell comes from the 31-bit position, which is
 // rounded down and at most 5 units low.  Where that hides a plane the ray has
 // just crossed, the next step finds the plane behind it and moves on with an
-// empty segment, so nothing is added to the wrong cell.
+// empty segment, so nothing is added to the wrong cell and no step is counted.
 template <bool TRACE, bool SPHERE, bool BRICKS>
 __device__ __forceinline__ void leaf_step(const KParams& kp, const TreeParams& tp, int64_t i, Ray& R,
                                           const uint32_t* stack, float sigma, float& w) {
@@ -1130,8 +1131,9 @@ constexpr int64_t DYNAMIC_MIN_RAYS = (int64_t)3 << 17;
 constexpr int64_t DYNAMIC_ALWAYS_RAYS = (int64_t)1 << 20;
 // Wavefronts of at least this many rays are also put in entry-cell order
 // (above): its fixed cost (a 5M-entry table per call) outweighs the gain on
-// smaller ones (depth-9 luminaire, 3M rays: 4.63 -> 4.70 ms with the order;
-// 9M rays: the same with and without).
+// smaller ones.  The line is where the two are even: depth-9 luminaire, 3M rays
+// 4.63 ms without and 4.70 with the order, 9M rays the same; depth-10, 16M
+// rays 46.0 and 40.8.
 constexpr int64_t ORDER_MIN_RAYS = (int64_t)1 << 23;
 
 template <bool TRACE>

@@ -62,7 +62,10 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
     return a;
 }
-// Arrive on a barrier of any CTA of the cluster.
+// Arrive on a barrier of any CTA of the cluster, at the default scope, which
+// orders this thread's accesses for its own CTA only: for what is complete where
+// the other CTA's tensor core reads it before the arrival is made (after a proxy
+// fence, a wait for the load, or tcgen05.wait::ld).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }

@@ -31,10 +31,21 @@
 // odd one's passes "this K-block has landed here" on to the even CTA); 2 lane
 // 0 TMA stores of the finished activation tiles; 3 lane 0 input tiles; 4..19
 // the epilogue (warp w reads TMEM lanes 32 (w % 4) .. +31 and a quarter of the
-// 32-column chunks).  Arrivals on the even CTA's barriers use the default
-// scope: what they announce has gone through a proxy fence or has landed, and
-// with the cluster scope each took so long that the chain of layers took 275
-// instead of 197 us without any work in it.  The epilogue writes its bf16 results into
+// 32-column chunks).
+//
+// The odd CTA's arrivals on the even one's barriers have the default scope,
+// .cta.  What each announces is complete, in the memory that the tensor core
+// reads, before it is made: kready, the K-block, waited for on wfull and passed
+// through fence.proxy.async; px, the input tile, whose TMA load has been waited
+// for on xfull; aready, the tile's bf16 values, written before
+// fence.proxy.async, and the accumulator, read before tcgen05.wait::ld and
+// tcgen05.fence::before_thread_sync.  No generic read of the other CTA's memory
+// follows.  Release and acquire at cluster scope cost (forward of 200,001
+// points / training step of 4096 x 128 / distillation at depth 7, us): none 230
+// / 1760 / 6773, px alone 231.5 / 1775 / 6940; releases on all 230 -> 244 /
+// 1760 -> 1880 / 7867 -> 8913.
+//
+// The epilogue writes its bf16 results into
 // the activation buffer in the layout a 128-byte-swizzled TMA load would
 // produce (row r's 16-byte chunk c at r * 128 + ((c ^ (r & 7)) * 16) of
 // its 64-column block), so the next layer's MMA and the TMA store read it
